@@ -165,9 +165,9 @@ __device__ __forceinline__ void tile_words(const SeedConst& sc, const uint64_t (
 // packed multiply fewer per block than scaling z = cos r after it is rounded.
 __device__ __forceinline__ void accum_block(uint4 w, float2 c, float2& acc_even, float2& acc_odd) {
     const Polar2 o = polar2(w);
-    const float2 rc = mul2<kPackO>(c, o.rr);
-    acc_even = fma2<kPackO>(o.cm, rc, acc_even);
-    acc_odd = fma2<kPackO>(o.sm, rc, acc_odd);
+    const float2 rc = mul2(c, o.rr);
+    acc_even = fma2(o.cm, rc, acc_even);
+    acc_odd = fma2(o.sm, rc, acc_odd);
 }
 
 // acc += c z for the Gaussians of the words w; accumulators are packed per block as

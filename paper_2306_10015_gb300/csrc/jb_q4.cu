@@ -171,7 +171,7 @@ __global__ void __maxnreg__(64) q4_perturb_kernel(const __grid_constant__ Q4Para
                                      static_cast<uint32_t>((blk0 + b + 1) >> 32));
             const Polar2 o = polar2(wcur);
             if (b + 1 < NB) wcur = wnext;
-            const float2 rc = mul2<kPackO>(eps2, o.rr);
+            const float2 rc = mul2(eps2, o.rr);
             float2 le, lo;
             switch (b) {
                 case 0: dequant_block<0>(pair, cw, le, lo); break;
@@ -183,8 +183,8 @@ __global__ void __maxnreg__(64) q4_perturb_kernel(const __grid_constant__ Q4Para
                 case 6: dequant_block<6>(pair, cw, le, lo); break;
                 default: dequant_block<7>(pair, cw, le, lo); break;
             }
-            wv[2 * b] = fma2<kPackO>(o.cm, rc, mul2<true>(le, s2));
-            wv[2 * b + 1] = fma2<kPackO>(o.sm, rc, mul2<true>(lo, s2));
+            wv[2 * b] = fma2(o.cm, rc, mul2(le, s2));
+            wv[2 * b + 1] = fma2(o.sm, rc, mul2(lo, s2));
         }
         // elements past the end of the segment do not count towards the maximum
         if (!full) {
@@ -212,7 +212,7 @@ __global__ void __maxnreg__(64) q4_perturb_kernel(const __grid_constant__ Q4Para
         for (int b = 0; b < NB; ++b) {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const float2 x = mul2<true>(wv[2 * b + h], inv2);
+                const float2 x = mul2(wv[2 * b + h], inv2);
                 const float2 y = __ffma2_rd(x, splat(0x1p-16f), splat(kQ4IdxBias));
                 const int ka = 4 * b + h, kb = 4 * b + h + 2;
                 ow[ka / 8] += q4_code(x.x, y.x, bucket) << (4 * (ka % 8));

@@ -11,19 +11,27 @@
 // Nothing here is written to memory on the hot path.
 //
 // Arithmetic of the transform (fp32, every rounding explicit):
-//   radius  u_a = 2^e f exactly, f in [3/4, 3/2), t = f - 1 exact; with
-//           q = -4t / (2 + t) (one rcp.approx), -2 ln(1 + t) = q + q w R(w),
-//           w = q^2, R a degree-2 minimax polynomial; L = -2 e ln 2 - 2 ln(1+t)
-//           with 2 ln 2 split hi + lo (Cody & Waite 1980) so e (2 ln 2)_hi is
-//           exact; r = sqrt.approx(L) (relative error below 1.1e-7 over
-//           every L the transform produces; one special-function operation
-//           where rsqrt.approx and a Newton step took four packed FP ones).
-//   angle   the 24-bit angle index splits into an octant (3 bits, handled
-//           exactly by reflection, swap and sign flips) and a 21-bit offset
-//           x in (0, 1) of the octant, sin(pi x / 4) and cos(pi x / 4) by
-//           minimax polynomials of degree 7 and 8 (relative error < 0.6 ulp
-//           for the sine, also near zero; 7.2e-8 for the cosine, which the
-//           octant keeps above 0.7).
+//   radius  u_a = 2^e f exactly, f in [1/2, 1), with sigma = 2(1 - f) exact and
+//           y = sigma / (2(1 + f)) (one rcp.approx):
+//           -2 ln f = 4 atanh(y) = sigma + y (sigma + w P(w)), w = y^2, P a degree-3
+//           minimax polynomial. The leading term is exact, so the error of the
+//           reciprocal enters only through the second term (at most 0.28 of the sum);
+//           u_a near 1 has e = 0 and keeps its relative accuracy.
+//           L = -2 ln f - e (2 ln 2) (2 ln 2 in fp32 is within 2.8e-9, so one product
+//           is enough); r = sqrt.approx(L) (relative error below 1.1e-7 over every L).
+//   angle   with t = x_b + 2^29, the angle is q pi/2 + (pi/4) x, q = t >> 30, x in
+//           (-1, 1) exact from the 22 bits below; sin and cos of (pi/4) x by minimax
+//           polynomials of degree 7 and 8 (relative error < 0.6 ulp for the sine, also
+//           near zero; 7.2e-8 for the cosine, which stays above 0.7). Odd q swaps them
+//           (and negates the sine), q >= 2 flips both: that sign goes to the radius.
+// Integers become floats by placing their bits under a constant exponent (one shift,
+// at most one mask, and a subtraction that the packed arithmetic does for two): an
+// integer-to-float conversion costs more issue slots than those. Against f in
+// [3/4, 3/2) with integer conversions, and an octant reflection with both signs applied
+// to the results, one pass over 1.3B bf16 elements went from 1653 to 1524 us (one pair)
+// and a K = 16 update of 125M fp32 elements from 2239 to 2123 us; it is also more
+// accurate: rms |dz| 4.75e-8 -> 4.69e-8, largest over 1.3e8 draws 8.0e-7 -> 7.5e-7,
+// joint worst case 8.7e-7 -> 8.2e-7.
 // Coefficients: fit_poly.py (Remez exchange). The transform is checked
 // against a double-precision evaluation of the same definition over all
 // radius words and all angle words (|dz| <= 1e-6).
@@ -39,14 +47,14 @@ constexpr uint32_t kPhiloxW0 = 0x9E3779B9u;
 constexpr uint32_t kPhiloxW1 = 0xBB67AE85u;
 
 // Polynomials (fit_poly.py).
-constexpr float kLogR0 = 0x1.5555b4p-6f, kLogR1 = 0x1.992aaap-11f, kLogR2 = 0x1.36ec6ap-15f;
+constexpr float kLogP0 = 0x1.5555p+0f, kLogP1 = 0x1.99d29ep-1f, kLogP2 = 0x1.1eb3a2p-1f,
+                kLogP3 = 0x1.1f0578p-1f;
 constexpr float kSinHi = 0x1.921fb6p-1f;   // pi/4 = hi + lo
 constexpr float kSinLo = -0x1.777a5cp-26f;
 constexpr float kSinS0 = -0x1.4abbbep-4f, kSinS1 = 0x1.465facp-9f, kSinS2 = -0x1.2db5cep-15f;
 constexpr float kCosC0 = -0x1.3bd3ccp-2f, kCosC1 = 0x1.03c1b0p-6f, kCosC2 = -0x1.55b2b6p-12f,
                 kCosC3 = 0x1.d4f7eep-19f;
-constexpr float kTwoLn2Hi = -0x1.62e4p+0f;       // -(2 ln 2) to 16 bits
-constexpr float kTwoLn2Lo = -0x1.7f7d1cp-19f;    // -(2 ln 2) - kTwoLn2Hi
+constexpr float kTwoLn2 = 0x1.62e430p+0f;
 
 struct Key {
     uint32_t k0, k1;       // machine id, low and high word
@@ -138,97 +146,72 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 
 __device__ __forceinline__ float2 splat(float a) { return make_float2(a, a); }
 
-// Two fp32 operations at once: one packed fp32x2 instruction, or two scalar ones.
-// Both round each component once to nearest, so the results are identical; the
-// choice only moves work between the FMA pipes (packed instructions share the
-// pipe that also runs the integer multiplies of Philox).
-template <bool PACK>
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-    if constexpr (PACK) return __ffma2_rn(a, b, c);
-    return make_float2(__fmaf_rn(a.x, b.x, c.x), __fmaf_rn(a.y, b.y, c.y));
-}
-template <bool PACK>
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
-    if constexpr (PACK) return __fmul2_rn(a, b);
-    return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));
-}
-template <bool PACK>
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-    if constexpr (PACK) return __fadd2_rn(a, b);
-    return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
-}
-
-#ifndef JB_PACK_RADIUS
-#define JB_PACK_RADIUS 1
-#endif
-#ifndef JB_PACK_ANGLE
-#define JB_PACK_ANGLE 1
-#endif
-#ifndef JB_PACK_OUT
-#define JB_PACK_OUT 1
-#endif
-constexpr bool kPackR = JB_PACK_RADIUS, kPackA = JB_PACK_ANGLE, kPackO = JB_PACK_OUT;
+// Two fp32 operations in one packed instruction, each rounded once to nearest.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 
 // Box-Muller of the two word pairs of a Philox block, (w.x, w.y) and (w.z, w.w), in
 // lockstep: every floating-point step is one packed fp32x2 instruction (two IEEE
-// round-to-nearest operations per issue slot), integer steps stay per pair. The
-// radius is carried with its sign flipped where a packed operation cannot negate an
-// operand (q = 4t/(2+t), L = 2 e ln 2 + 2 ln(1+t) = ln u_a^-2 negated, -r) and
-// the sign is restored in the final sign masks; round-to-nearest is odd-symmetric,
-// so no rounding differs from the unflipped formulas.
-// Polar form: rr = (-r of pair A, -r of pair B); cm, sm = the signed cosines and sines
-// (sign flips of the negated radius included), so z_even = cm rr, z_odd = sm rr.
+// round-to-nearest operations per issue slot), integer steps stay per pair.
+// Polar form: rr = the radii of pair A and pair B, with the sign of the angle's half
+// turn; cm, sm = cosines and sines up to that sign, so z_even = cm rr, z_odd = sm rr.
 struct Polar2 {
     float2 rr, cm, sm;
 };
 
+// The word hi : lo shifted right by n, low half: one instruction that moves bits of lo
+// into the mantissa and puts an exponent above them.
+__device__ __forceinline__ float shift_under(uint32_t hi, uint32_t lo, int n) {
+    return __uint_as_float(__funnelshift_r(lo, hi, n));
+}
+
+__device__ __forceinline__ float masked(uint32_t bits, uint32_t keep, uint32_t set) {
+    return __uint_as_float((bits & keep) | set);
+}
+
 __device__ __forceinline__ Polar2 polar2(uint4 w) {
     // ---- radius ----
-    const uint32_t ybA = __float_as_uint(__uint2float_rn((w.x & 0xFFFFFE00u) | 0x100u));
-    const uint32_t ybB = __float_as_uint(__uint2float_rn((w.z & 0xFFFFFE00u) | 0x100u));
-    const int32_t ixA = static_cast<int32_t>(ybA - 0x4F400000u);
-    const int32_t ixB = static_cast<int32_t>(ybB - 0x4F400000u);
-    const float2 f = make_float2(
-        __uint_as_float((static_cast<uint32_t>(ixA) & 0x7FFFFFu) + 0x3F400000u),
-        __uint_as_float((static_cast<uint32_t>(ixB) & 0x7FFFFFu) + 0x3F400000u));
-    const float2 t = add2<kPackR>(f, splat(-1.0f));
-    const float2 d = fma2<kPackR>(t, splat(0.25f), splat(0.5f));      // (2 + t) / 4
-    const float2 q = mul2<kPackR>(t, make_float2(rcp_approx(d.x), rcp_approx(d.y)));  // 4t/(2+t)
-    const float2 ww = mul2<kPackR>(q, q);
-    float2 p = fma2<kPackR>(ww, splat(kLogR2), splat(kLogR1));
-    p = fma2<kPackR>(ww, p, splat(kLogR0));
-    const float2 lp = fma2<kPackR>(q, mul2<kPackR>(ww, p), q);          // 2 ln(1 + t)
-    const float2 fe = make_float2(__int2float_rn(ixA >> 23), __int2float_rn(ixB >> 23));
-    const float2 l_lo = fma2<kPackR>(fe, splat(-kTwoLn2Lo), lp);
-    // e (2 ln 2)_hi is exact, so L is l_hi + l_lo rounded once
-    const float2 L = fma2<kPackR>(fe, splat(-kTwoLn2Hi), l_lo);         // -(-2 ln u_a)
-    Polar2 o;
-    o.rr = make_float2(-sqrt_approx(-L.x), -sqrt_approx(-L.y));       // -r
+    // 1 + (x_a >> 9) 2^-23, less 1 - 2^-24: u_a, exact
+    const float2 u = add2(make_float2(shift_under(0x7Fu, w.x, 9), shift_under(0x7Fu, w.z, 9)),
+                          splat(-0x1.fffffep-1f));
+    const uint32_t uA = __float_as_uint(u.x), uB = __float_as_uint(u.y);
+    const float2 f = make_float2(masked(uA, 0x7FFFFFu, 0x3F000000u), masked(uB, 0x7FFFFFu, 0x3F000000u));
+    // 2^23 + biased exponent, less 2^23 + 126: e, exact
+    const float2 e = add2(make_float2(shift_under(0x4B000000u >> 9, uA, 23),
+                                      shift_under(0x4B000000u >> 9, uB, 23)), splat(-8388734.0f));
+    const float2 sg = fma2(f, splat(-2.0f), splat(2.0f));             // 2(1 - f), exact
+    const float2 d = fma2(f, splat(2.0f), splat(2.0f));
+    const float2 y = mul2(sg, make_float2(rcp_approx(d.x), rcp_approx(d.y)));  // (1 - f) / (1 + f)
+    const float2 ww = mul2(y, y);
+    float2 p = fma2(ww, splat(kLogP3), splat(kLogP2));
+    p = fma2(ww, p, splat(kLogP1));
+    p = fma2(ww, p, splat(kLogP0));
+    const float2 lf = fma2(y, fma2(ww, p, sg), sg);                   // -2 ln f
+    const float2 L = fma2(e, splat(-kTwoLn2), lf);                    // -2 ln u_a
 
     // ---- angle ----
-    const int32_t waA = static_cast<int32_t>(((w.y << 2) & 0xFFFFFC00u) | 0x200u);
-    const int32_t waB = static_cast<int32_t>(((w.w << 2) & 0xFFFFFC00u) | 0x200u);
-    const float2 x = make_float2(__fmul_rn(fabsf(__int2float_rn(waA)), 0x1p-31f),
-                                 __fmul_rn(fabsf(__int2float_rn(waB)), 0x1p-31f));
-    const float2 y = mul2<kPackA>(x, x);
-    float2 ps = fma2<kPackA>(y, splat(kSinS2), splat(kSinS1));
-    ps = fma2<kPackA>(y, ps, splat(kSinS0));
-    ps = fma2<kPackA>(y, ps, splat(kSinLo));
-    const float2 S = fma2<kPackA>(x, splat(kSinHi), mul2<kPackA>(x, ps));
-    float2 pc = fma2<kPackA>(y, splat(kCosC3), splat(kCosC2));
-    pc = fma2<kPackA>(y, pc, splat(kCosC1));
-    pc = fma2<kPackA>(y, pc, splat(kCosC0));
-    const float2 C = fma2<kPackA>(y, pc, splat(1.0f));
-    // octant bits o2 o1 o0 = word bits 31..29: |cos| and |sin| swap when o0 ^ o1;
-    // cos < 0 when o1 ^ o2, sin < 0 when o2; one more flip for the negated radius
-    const uint32_t tA = w.y ^ (w.y << 1), tB = w.w ^ (w.w << 1);
+    const uint32_t tA = w.y + 0x20000000u, tB = w.w + 0x20000000u;
+    // [1, 2) from bits 29 .. 8 and a last bit for the half: 2 (.) - 3 = x, exact
+    const float2 x = fma2(make_float2(masked(tA >> 7, 0x7FFFFEu, 0x3F800001u),
+                                      masked(tB >> 7, 0x7FFFFEu, 0x3F800001u)),
+                          splat(2.0f), splat(-3.0f));
+    const float2 xx = mul2(x, x);
+    float2 ps = fma2(xx, splat(kSinS2), splat(kSinS1));
+    ps = fma2(xx, ps, splat(kSinS0));
+    ps = fma2(xx, ps, splat(kSinLo));
+    const float2 S = fma2(x, splat(kSinHi), mul2(x, ps));
+    float2 pc = fma2(xx, splat(kCosC3), splat(kCosC2));
+    pc = fma2(xx, pc, splat(kCosC1));
+    pc = fma2(xx, pc, splat(kCosC0));
+    const float2 C = fma2(xx, pc, splat(1.0f));
     const bool swA = (tA & 0x40000000u) != 0u, swB = (tB & 0x40000000u) != 0u;
-    o.cm = make_float2(
-        __uint_as_float(__float_as_uint(swA ? S.x : C.x) ^ (tA & 0x80000000u) ^ 0x80000000u),
-        __uint_as_float(__float_as_uint(swB ? S.y : C.y) ^ (tB & 0x80000000u) ^ 0x80000000u));
-    o.sm = make_float2(
-        __uint_as_float(__float_as_uint(swA ? C.x : S.x) ^ (w.y & 0x80000000u) ^ 0x80000000u),
-        __uint_as_float(__float_as_uint(swB ? C.y : S.y) ^ (w.w & 0x80000000u) ^ 0x80000000u));
+    Polar2 o;
+    o.rr = make_float2(
+        __uint_as_float(__float_as_uint(sqrt_approx(L.x)) ^ (tA & 0x80000000u)),
+        __uint_as_float(__float_as_uint(sqrt_approx(L.y)) ^ (tB & 0x80000000u)));
+    o.cm = make_float2(swA ? -S.x : C.x, swB ? -S.y : C.y);
+    o.sm = make_float2(swA ? C.x : S.x, swB ? C.y : S.y);
     return o;
 }
 
@@ -240,8 +223,8 @@ struct GaussPair {
 __device__ __forceinline__ GaussPair box_muller2(uint4 w) {
     const Polar2 o = polar2(w);
     GaussPair g;
-    g.even = mul2<kPackO>(o.cm, o.rr);
-    g.odd = mul2<kPackO>(o.sm, o.rr);
+    g.even = mul2(o.cm, o.rr);
+    g.odd = mul2(o.sm, o.rr);
     return g;
 }
 
