@@ -22,9 +22,7 @@ namespace {
 
 constexpr uint64_t kMaxIndex = 1ull << 62;  // global element indices stay below this
 
-struct Seg {
-    uint64_t ptr, fo, n;
-};
+using jb::Seg;
 
 size_t elem_size(int dtype) { return dtype == JB_F32 ? 4 : 2; }
 
@@ -73,15 +71,15 @@ int collect_segments(const jb_segment* segs, int n_segs, int dtype, std::vector<
     return JB_OK;
 }
 
-// Fills params.segs / n_segs / n_vec with segments [first, first + count).
-template <typename P>
-void pack_segments(const std::vector<Seg>& segs, size_t first, size_t count, int dtype, P& params) {
+// Fills params with segments [first, first + count).
+void pack_segments(const std::vector<Seg>& segs, size_t first, size_t count, int dtype,
+                   jb::SumParams& params) {
     const uint64_t E = static_cast<uint64_t>(elems_per_vec(dtype));
     const uint64_t es = elem_size(dtype);
     uint64_t vec = 0;
     for (size_t i = 0; i < count; ++i) {
         const Seg& s = segs[first + i];
-        jb::SegParam& g = params.segs[i];
+        jb::SumSegParam& g = params.segs[i];
         const uint64_t v_begin = s.fo / E;
         const uint64_t v_end = (s.fo + s.n + E - 1) / E;
         // 16-byte vectors of the segment line up with element groups whose global
@@ -97,14 +95,9 @@ void pack_segments(const std::vector<Seg>& segs, size_t first, size_t count, int
     params.n_vec = vec;
 }
 
-jb::SeedParam seed_param(const jb_seed& s, float coef) {
-    jb::SeedParam p;
-    p.k0 = static_cast<uint32_t>(s.machine_id);
-    p.k1 = static_cast<uint32_t>(s.machine_id >> 32);
-    p.step = s.step;
-    p.sample = s.sample_id;
-    p.coef = coef;
-    return p;
+jb::SeedRaw seed_raw(const jb_seed& s) {
+    return {static_cast<uint32_t>(s.machine_id), static_cast<uint32_t>(s.machine_id >> 32), s.step,
+            s.sample_id};
 }
 
 bool seed_less(const jb_seed& a, const jb_seed& b) {
@@ -141,16 +134,9 @@ int perturb_impl(const jb_segment* segs, int n_segs, int dtype, jb_seed seed, fl
     if (rc != JB_OK) return rc;
     if (!std::isfinite(eps)) return JB_ERR_INVALID_ARG;
     if (v.empty()) return JB_OK;
-    static thread_local jb::PerturbParams params;  // ~32 KB: keep it off the stack
-    params.n_seeds = 1;
-    params.seeds[0] = seed_param(seed, eps);
-    for (size_t first = 0; first < v.size(); first += jb::kMaxSegsPerturb) {
-        const size_t count = std::min<size_t>(jb::kMaxSegsPerturb, v.size() - first);
-        pack_segments(v, first, count, dtype, params);
-        rc = cuda_status(jb::launch_perturb(params, dtype, grid_ctas, stream));
-        if (rc != JB_OK) return rc;
-    }
-    return JB_OK;
+    const jb::SeedRaw raw = seed_raw(seed);
+    jb::Job job{jb::kPerturb, dtype, &raw, &eps, 1, nullptr, 0, false, grid_ctas, stream};
+    return cuda_status(jb::enqueue(job, v.data(), nullptr, v.size()));
 }
 
 int update_impl(const jb_segment* segs, int n_segs, int dtype, const jb_seed* seeds,
@@ -174,24 +160,19 @@ int update_impl(const jb_segment* segs, int n_segs, int dtype, const jb_seed* se
     for (int k = 1; k < K; ++k)
         if (seed_equal(seeds[order[k - 1]], seeds[order[k]])) return JB_ERR_DUPLICATE_SEED;
 
-    static thread_local jb::UpdateParams params;
-    params.n_seeds = static_cast<uint32_t>(K);
+    std::vector<jb::SeedRaw> raw(static_cast<size_t>(K));
+    std::vector<float> coef(static_cast<size_t>(K));
     for (int k = 0; k < K; ++k) {
         const int i = order[k];
         const double c = -static_cast<double>(lr) * dequantize(q[i], static_cast<double>(qscale)) /
                          static_cast<double>(denom);
-        const float cf = static_cast<float>(c);
-        if (!std::isfinite(cf)) return JB_ERR_RANGE;
-        params.seeds[k] = seed_param(seeds[i], cf);
+        coef[k] = static_cast<float>(c);
+        if (!std::isfinite(coef[k])) return JB_ERR_RANGE;
+        raw[k] = seed_raw(seeds[i]);
     }
     if (v.empty()) return JB_OK;
-    for (size_t first = 0; first < v.size(); first += jb::kMaxSegsUpdate) {
-        const size_t count = std::min<size_t>(jb::kMaxSegsUpdate, v.size() - first);
-        pack_segments(v, first, count, dtype, params);
-        rc = cuda_status(jb::launch_update(params, dtype, grid_ctas, stream));
-        if (rc != JB_OK) return rc;
-    }
-    return JB_OK;
+    jb::Job job{jb::kUpdate, dtype, raw.data(), coef.data(), K, nullptr, 0, false, grid_ctas, stream};
+    return cuda_status(jb::enqueue(job, v.data(), nullptr, v.size()));
 }
 
 // Destination table for src: same numel and flat offsets, element-aligned; each
@@ -257,7 +238,8 @@ int general_impl(const jb_segment* segs, const jb_segment* dsts, int n_segs, int
     if (total > 0 && (seeds == nullptr || q == nullptr)) return JB_ERR_INVALID_ARG;
 
     // every group in canonical order, with its coefficients
-    std::vector<jb::SeedParam> all(static_cast<size_t>(total));
+    std::vector<jb::SeedRaw> raw(static_cast<size_t>(total));
+    std::vector<float> coef(static_cast<size_t>(total));
     std::vector<int> sizes;
     long long base = 0;
     for (int g = 0; g < n_groups; ++g) {
@@ -274,7 +256,8 @@ int general_impl(const jb_segment* segs, const jb_segment* dsts, int n_segs, int
                              static_cast<double>(denom[g]);
             const float cf = static_cast<float>(c);
             if (!std::isfinite(cf)) return JB_ERR_RANGE;
-            all[static_cast<size_t>(base + k)] = seed_param(seeds[i], cf);
+            raw[static_cast<size_t>(base + k)] = seed_raw(seeds[i]);
+            coef[static_cast<size_t>(base + k)] = cf;
         }
         base += K;
         if (K > 0) sizes.push_back(K);  // an empty group changes nothing
@@ -285,56 +268,30 @@ int general_impl(const jb_segment* segs, const jb_segment* dsts, int n_segs, int
         sizes.clear();  // a pure copy: one launch with no group
     }
 
-    static thread_local jb::GeneralParams params;
-    const uint64_t E = static_cast<uint64_t>(elems_per_vec(dtype));
-    const uint64_t es = elem_size(dtype);
     // groups in launches of at most kMaxSeedsPerLaunch pairs / kMaxGroupsPerLaunch groups;
     // after the first launch the destination holds the running value
+    std::vector<Seg> from(v);
+    std::vector<uint16_t> ends;
     size_t g0 = 0;
     long long s0 = 0;
-    bool first = true;
     do {
         size_t g1 = g0;
         long long n = 0;
+        ends.clear();
         while (g1 < sizes.size() && g1 - g0 < static_cast<size_t>(jb::kMaxGroupsPerLaunch) &&
-               n + sizes[g1] <= jb::kMaxSeedsPerLaunch)
+               n + sizes[g1] <= jb::kMaxSeedsPerLaunch) {
             n += sizes[g1++];
-        params.n_seeds = static_cast<uint32_t>(n);
-        params.n_groups = static_cast<uint32_t>(g1 - g0);
-        long long acc = 0;
-        for (size_t g = g0; g < g1; ++g) {
-            acc += sizes[g];
-            params.group_end[g - g0] = static_cast<uint16_t>(acc);
+            ends.push_back(static_cast<uint16_t>(n));
         }
-        for (long long k = 0; k < n; ++k) params.seeds[k] = all[static_cast<size_t>(s0 + k)];
         const bool last = g1 >= sizes.size();
         // write_src comes with one group only (jb_apply_updates_from): one launch round
-        params.write_src = (write_src && last) ? 1u : 0u;
-        for (size_t first_seg = 0; first_seg < v.size(); first_seg += jb::kMaxSegsGeneral) {
-            const size_t count = std::min<size_t>(jb::kMaxSegsGeneral, v.size() - first_seg);
-            uint64_t vec = 0;
-            for (size_t i = 0; i < count; ++i) {
-                const Seg& sg = v[first_seg + i];
-                const uint64_t src_ptr = first ? sg.ptr : dptr[first_seg + i];
-                const uint64_t dst_ptr = dptr[first_seg + i];
-                jb::SegParamOut& g = params.segs[i];
-                const bool aligned = ((src_ptr - sg.fo * es) & 15ull) == 0 &&
-                                     ((dst_ptr - sg.fo * es) & 15ull) == 0;
-                g.ptr = src_ptr | (aligned ? 1ull : 0ull);
-                g.dst = dst_ptr;
-                g.fo = sg.fo;
-                g.n = sg.n;
-                g.vec0 = vec;
-                vec += (sg.fo + sg.n + E - 1) / E - sg.fo / E;
-            }
-            params.n_segs = static_cast<uint32_t>(count);
-            params.n_vec = vec;
-            rc = cuda_status(jb::launch_general(params, dtype, grid_ctas, stream));
-            if (rc != JB_OK) return rc;
-        }
+        jb::Job job{jb::kGeneral, dtype, raw.data() + s0, coef.data() + s0, static_cast<int>(n),
+                    ends.data(), static_cast<int>(ends.size()), write_src && last, grid_ctas, stream};
+        rc = cuda_status(jb::enqueue(job, from.data(), dptr.data(), from.size()));
+        if (rc != JB_OK) return rc;
+        for (size_t i = 0; i < from.size(); ++i) from[i].ptr = dptr[i];
         s0 += n;
         g0 = g1;
-        first = false;
     } while (g0 < sizes.size());
     return JB_OK;
 }
@@ -397,10 +354,9 @@ int checksum_impl(const jb_segment* segs, int n_segs, int dtype, uint64_t* d_out
     if (reinterpret_cast<uint64_t>(d_out) & 7ull) return JB_ERR_MISALIGNED;
     rc = cuda_status(cudaMemsetAsync(d_out, 0, sizeof(uint64_t), stream));
     if (rc != JB_OK) return rc;
-    static thread_local jb::PerturbParams params;
-    params.n_seeds = 0;
-    for (size_t first = 0; first < v.size(); first += jb::kMaxSegsPerturb) {
-        const size_t count = std::min<size_t>(jb::kMaxSegsPerturb, v.size() - first);
+    static thread_local jb::SumParams params;  // ~32 KB: keep it off the stack
+    for (size_t first = 0; first < v.size(); first += jb::kMaxSegsSum) {
+        const size_t count = std::min<size_t>(jb::kMaxSegsSum, v.size() - first);
         pack_segments(v, first, count, dtype, params);
         rc = cuda_status(jb::launch_checksum(params, dtype, reinterpret_cast<unsigned long long*>(d_out),
                                              grid_ctas, stream));
@@ -449,10 +405,13 @@ int perturb_q4_impl(const jb_q4_segment* segs, int n_segs, jb_seed seed, float e
     }
     if (v.empty()) return JB_OK;
     static thread_local jb::Q4Params params;
-    params.seed = seed_param(seed, eps);
+    params.seed = seed_raw(seed);
+    params.eps = eps;
     for (size_t first = 0; first < v.size(); first += jb::kMaxSegsQ4) {
         const size_t count = std::min<size_t>(jb::kMaxSegsQ4, v.size() - first);
         uint64_t unit = 0;
+        params.block_hi = static_cast<uint32_t>(v[first].fo >> 34);
+        params.one_hi = 1;
         for (size_t i = 0; i < count; ++i) {
             const Q& q = v[first + i];
             jb::SegParamQ4& g = params.segs[i];
@@ -461,6 +420,9 @@ int perturb_q4_impl(const jb_q4_segment* segs, int n_segs, jb_seed seed, float e
             g.fo = q.fo;
             g.n = q.n;
             g.unit0 = unit;
+            // (a unit past the end of a tensor draws nothing that is kept)
+            if ((q.fo >> 34) != params.block_hi || ((q.fo + q.n - 1) >> 34) != params.block_hi)
+                params.one_hi = 0;
             unit += jb::kQ4UnitsPerBlock * ((q.n + 63) / 64);  // whole 64-element blocks
         }
         params.n_segs = static_cast<uint32_t>(count);
@@ -525,7 +487,7 @@ JB_EXPORT int jb_debug_philox(jb_seed seed, uint64_t first_block, uint64_t n_blo
     if (n_blocks > 0 && d_out == nullptr) return JB_ERR_INVALID_ARG;
     if (n_blocks > (1ull << 38)) return JB_ERR_INVALID_ARG;
     if (reinterpret_cast<uint64_t>(d_out) & 15ull) return JB_ERR_MISALIGNED;  // one 16-byte store per block
-    return cuda_status(jb::launch_debug_philox(seed_param(seed, 0.0f), first_block, n_blocks, d_out,
+    return cuda_status(jb::launch_debug_philox(seed_raw(seed), first_block, n_blocks, d_out,
                                                stream));
 }
 
@@ -534,7 +496,7 @@ JB_EXPORT int jb_debug_philox_fold(jb_seed seed, uint64_t first_block, uint64_t 
     if (d_out == nullptr) return JB_ERR_INVALID_ARG;
     if (n_blocks > (1ull << 46) || first_block > (1ull << 60)) return JB_ERR_INVALID_ARG;
     if (reinterpret_cast<uint64_t>(d_out) & 3ull) return JB_ERR_MISALIGNED;
-    return cuda_status(jb::launch_debug_philox_fold(seed_param(seed, 0.0f), first_block, n_blocks,
+    return cuda_status(jb::launch_debug_philox_fold(seed_raw(seed), first_block, n_blocks,
                                                     d_out, stream));
 }
 
@@ -543,7 +505,7 @@ JB_EXPORT int jb_debug_gaussian(jb_seed seed, uint64_t first_elem, uint64_t n, f
     if (n > 0 && d_out == nullptr) return JB_ERR_INVALID_ARG;
     if (n > (1ull << 38) || first_elem > kMaxIndex - n) return JB_ERR_INVALID_ARG;
     if (reinterpret_cast<uint64_t>(d_out) & 3ull) return JB_ERR_MISALIGNED;
-    return cuda_status(jb::launch_debug_gaussian(seed_param(seed, 0.0f), first_elem, n, d_out, stream));
+    return cuda_status(jb::launch_debug_gaussian(seed_raw(seed), first_elem, n, d_out, stream));
 }
 
 JB_EXPORT int jb_debug_box_muller(const uint32_t* d_words, uint64_t n_pairs, float* d_out,

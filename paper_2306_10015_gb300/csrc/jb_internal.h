@@ -1,13 +1,23 @@
 // jb_internal.h -- launch descriptors shared by the C ABI (jb_capi.cpp) and
-// the kernels (jb_kernels.cu). Not part of the public interface.
+// the kernels (jb_kernels.cu, jb_q4.cu). Not part of the public interface.
 //
 // A launch carries its whole work description in the kernel parameter space
-// (up to 32,764 bytes on sm_70 and later): the K (seed, coefficient) pairs are
-// read with warp-uniform indices from the constant bank, and the segment table
-// maps a flat "vector" index to a tensor. A vector is 16 bytes of one segment
-// whose elements are aligned to Philox blocks in global index: 4 fp32 or 8
-// bf16 elements. Segment s owns the global vectors floor(fo / E) ..
-// ceil((fo + n) / E) - 1; its first one is launch vector vec0.
+// (up to 32,764 bytes on sm_70 and later): the K (seed, coefficient) pairs, read
+// with warp-uniform indices from the constant bank, then the segment table. The two
+// share one block of bytes, so that few pairs leave room for more segments.
+//
+// Work is cut into 16-byte "vectors" of one segment whose elements are aligned to
+// Philox blocks in global index (4 fp32 or 8 bf16 elements), and vectors into warp
+// tiles of 32 V of them. A tile lies in one segment: segment s owns tiles
+// tile0 .. (tile0 of the next) - 1, and a sentinel entry after the last one holds
+// the number of tiles, so a tile's segment is the last entry whose tile0 is not
+// above it.
+//
+// All global indices of a launch agree in the high word of their Philox block
+// index: the host cuts segments at multiples of 2^33 elements and puts those of
+// different high words into different launches. Block counters are therefore 32-bit
+// in the kernels, and the whole first round and half of the second are constants of
+// the pair (jb_rng.cuh).
 #pragma once
 #include <cstdint>
 
@@ -15,73 +25,105 @@
 
 namespace jb {
 
-#ifndef JB_THREADS
-#define JB_THREADS 512
-#endif
-constexpr int kThreads = JB_THREADS;   // threads per CTA
+constexpr int kThreads = 512;  // threads per CTA of the checksum and the generator alone
 constexpr int kMaxSeedsPerLaunch = 512;
-constexpr int kMaxSegsUpdate = 700;    // 16 + 512 * 20 + 700 * 32 bytes
-constexpr int kMaxSegsPerturb = 1000;  // 16 + 24 + 1000 * 32 bytes
+constexpr int kMaxGroupsPerLaunch = 512;
+constexpr uint64_t kPieceElems = 1ull << 33;  // segments are cut at multiples of this index
 
-struct SeedParam {
+// Philox4x32 round multipliers and key increments (Salmon et al. 2011).
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u;
+constexpr uint32_t kPhiloxM1 = 0xCD9E8D57u;
+constexpr uint32_t kPhiloxW0 = 0x9E3779B9u;
+constexpr uint32_t kPhiloxW1 = 0xBB67AE85u;
+
+// Seed s of the method: the key and the upper half of the counter.
+struct SeedRaw {
     uint32_t k0, k1;        // machine id (lo, hi)
     uint32_t step, sample;  // counter words 2 and 3
-    float coef;             // c_k (update) or eps (perturb)
 };
 
+// A pair as the kernels read it: the words of Philox4x32-10 that do not depend on the
+// low word of the block index (philox_block in jb_rng.cuh), and the scale.
+struct alignas(16) SeedParam {
+    uint32_t c2;       // round 1: x2 = hi(M0 b_lo) ^ c2
+    uint32_t c0;       // round 2: x0 = hi(M1 x2) ^ c0
+    uint32_t n2, n3;   // round 2: x2 = lo(M0 b_lo) ^ n2, x3 = n3
+    uint32_t k0, k1;   // keys of round 3
+    float coef;        // c_k (update) or eps (perturb)
+    uint32_t ends_group;  // general update: round to the storage type after this pair
+};
+
+__host__ __device__ inline SeedParam seed_param(const SeedRaw& s, uint32_t block_hi, float coef) {
+    const uint64_t a = static_cast<uint64_t>(kPhiloxM1) * s.step;
+    const uint32_t x0 = static_cast<uint32_t>(a >> 32) ^ block_hi ^ s.k0;  // after round 1
+    const uint64_t p = static_cast<uint64_t>(kPhiloxM0) * x0;
+    SeedParam r;
+    r.c2 = s.sample ^ s.k1;
+    r.c0 = static_cast<uint32_t>(a) ^ (s.k0 + kPhiloxW0);
+    r.n2 = static_cast<uint32_t>(p >> 32) ^ (s.k1 + kPhiloxW1);
+    r.n3 = static_cast<uint32_t>(p);
+    r.k0 = s.k0 + 2u * kPhiloxW0;
+    r.k1 = s.k1 + 2u * kPhiloxW1;
+    r.coef = coef;
+    r.ends_group = 0;
+    return r;
+}
+
 struct SegParam {
+    uint64_t base;   // device address of the segment's first window (its element `head` is element 0)
+    uint64_t end;    // elements of the segment are [head, end) of its windows
+    uint32_t blk0;   // low word of the Philox block index of the first window
+    uint32_t tile0;  // first tile
+    uint32_t head;   // elements of the first window before the segment (0 .. E - 1)
+    uint32_t full;   // vectors [head ? 1 : 0, full) take 16-byte accesses; 0: none does
+};
+
+struct SegParamOut : SegParam {
+    uint64_t dst;    // destination address of the first window
+};
+
+template <typename SEG, int BYTES>
+struct Launch {
+    using Seg = SEG;
+    static constexpr int kBytes = BYTES;
+    uint32_t n_seeds;
+    uint32_t n_segs;
+    uint32_t n_tiles;
+    uint32_t span;       // consecutive tiles that a warp takes at a time
+    uint32_t write_src;  // write the result to the source too
+    uint32_t seg_at;     // byte offset of the segment table in `data`; the pairs are at 0
+    alignas(16) unsigned char data[BYTES];
+};
+
+constexpr int kParamBytes = 32704;
+static_assert(sizeof(Launch<SegParam, kParamBytes>) <= 32764, "launch exceeds the parameter space");
+
+// A checked segment: element i at ptr + i sizeof(T) has global index fo + i.
+struct Seg {
+    uint64_t ptr, fo, n;
+};
+
+// Checksum: no pairs, and windows keep their 64-bit index.
+constexpr int kMaxSegsSum = 1000;
+
+struct SumSegParam {
     uint64_t ptr;   // device address; bit 0 set when the 16-byte vector path applies
     uint64_t fo;    // global index of element 0
     uint64_t n;     // elements
     uint64_t vec0;  // first launch vector of this segment
 };
 
-template <int MAXK, int MAXS>
-struct LaunchParams {
-    uint32_t n_seeds;
+struct SumParams {
     uint32_t n_segs;
     uint64_t n_vec;  // vectors in this launch
-    SeedParam seeds[MAXK];
-    SegParam segs[MAXS];
+    SumSegParam segs[kMaxSegsSum];
 };
 
-using UpdateParams = LaunchParams<kMaxSeedsPerLaunch, kMaxSegsUpdate>;
-using PerturbParams = LaunchParams<1, kMaxSegsPerturb>;
-
-static_assert(sizeof(UpdateParams) <= 32764, "update launch exceeds the parameter space");
-static_assert(sizeof(PerturbParams) <= 32764, "perturb launch exceeds the parameter space");
-
-// Generalised update: reads segment `ptr`, writes segment `dst` (and `ptr` too when
-// write_src), and applies the seeds in groups, rounding to the storage type after
-// each group: group g covers seeds [group_end[g - 1], group_end[g]).
-constexpr int kMaxGroupsPerLaunch = 512;
-constexpr int kMaxSegsGeneral = 512;
-
-struct SegParamOut {
-    uint64_t ptr;   // source; bit 0 set when source and destination take the vector path
-    uint64_t dst;   // destination
-    uint64_t fo;
-    uint64_t n;
-    uint64_t vec0;
-};
-
-struct GeneralParams {
-    uint32_t n_seeds;
-    uint32_t n_segs;
-    uint64_t n_vec;
-    uint32_t n_groups;
-    uint32_t write_src;
-    SeedParam seeds[kMaxSeedsPerLaunch];
-    uint16_t group_end[kMaxGroupsPerLaunch];
-    SegParamOut segs[kMaxSegsGeneral];
-};
-
-static_assert(sizeof(GeneralParams) <= 32764, "general launch exceeds the parameter space");
+static_assert(sizeof(SumParams) <= 32764, "checksum launch exceeds the parameter space");
 
 // 4-bit weights: codes (two per byte, element 2i in the low nibble) and one fp32
-// scale per 64 elements. Work unit: 16 elements (8 code bytes); a segment owns
-// units [unit0, unit0 + ceil(n / 64) * 4), so a 64-element block is always four
-// consecutive units, handled by four consecutive lanes.
+// scale per 64 elements. A segment owns units [unit0, unit0 + units), kQ4UnitsPerBlock
+// consecutive units per 64-element block (jb_q4.h).
 constexpr int kMaxSegsQ4 = 800;
 
 struct SegParamQ4 {
@@ -93,8 +135,11 @@ struct SegParamQ4 {
 };
 
 struct Q4Params {
-    SeedParam seed;  // coef = eps
+    SeedRaw seed;
+    float eps;
     uint32_t n_segs;
+    uint32_t block_hi;   // high word of the first block index of the launch
+    uint32_t one_hi;     // every block index of the launch has that high word
     uint64_t n_units;
     SegParamQ4 segs[kMaxSegsQ4];
 };
@@ -106,17 +151,35 @@ void q4_levels_host(float out[16]);
 
 enum DType { kF32 = 0, kBF16 = 1 };
 
-// Launchers (jb_kernels.cu). grid_ctas <= 0 selects the persistent grid.
-cudaError_t launch_update(const UpdateParams& p, int dtype, int grid_ctas, cudaStream_t s);
-cudaError_t launch_perturb(const PerturbParams& p, int dtype, int grid_ctas, cudaStream_t s);
-cudaError_t launch_general(const GeneralParams& p, int dtype, int grid_ctas, cudaStream_t s);
-cudaError_t launch_checksum(const PerturbParams& p, int dtype, unsigned long long* out,
-                            int grid_ctas, cudaStream_t s);
-cudaError_t launch_debug_philox(SeedParam seed, uint64_t first_block, uint64_t n_blocks,
+// What a launch runs: PerturbParameters (one pair, theta + eps z as one fused
+// multiply-add), the in-place update, or the general update (source to destination,
+// groups). One pair in one group takes the one-pair kernel in both updates.
+enum Work { kPerturb = 0, kUpdate = 1, kGeneral = 2 };
+
+struct Job {
+    Work work;
+    int dtype;
+    const SeedRaw* seeds;  // in canonical order (within each group)
+    const float* coef;
+    int n_seeds;
+    const uint16_t* group_end;  // general update: group g is the pairs up to group_end[g]
+    int n_groups;
+    bool write_src;
+    int grid_ctas;  // <= 0: the persistent grid
+    cudaStream_t stream;
+};
+
+// Packs the segments into launches of the job and enqueues them. dst: the general
+// update's destinations, one per segment (n_segs > 0).
+cudaError_t enqueue(const Job& job, const Seg* segs, const uint64_t* dst, size_t n_segs);
+
+cudaError_t launch_checksum(const SumParams& p, int dtype, unsigned long long* out, int grid_ctas,
+                            cudaStream_t s);
+cudaError_t launch_debug_philox(SeedRaw seed, uint64_t first_block, uint64_t n_blocks,
                                 uint32_t* out, cudaStream_t s);
-cudaError_t launch_debug_philox_fold(SeedParam seed, uint64_t first_block, uint64_t n_blocks,
+cudaError_t launch_debug_philox_fold(SeedRaw seed, uint64_t first_block, uint64_t n_blocks,
                                      uint32_t* out, cudaStream_t s);
-cudaError_t launch_debug_gaussian(SeedParam seed, uint64_t first, uint64_t n, float* out,
+cudaError_t launch_debug_gaussian(SeedRaw seed, uint64_t first, uint64_t n, float* out,
                                   cudaStream_t s);
 cudaError_t launch_debug_box_muller(const uint32_t* words, uint64_t n_pairs, float* out,
                                     cudaStream_t s);

@@ -93,8 +93,10 @@ __device__ __forceinline__ void dequant_block(const float2* pair, const uint32_t
 
 constexpr int kThreadsQ4 = 512;
 
-// 64 registers: two CTAs per SM (8 bytes spilled), measured 2.7% faster than the
-// compiler's 70 registers and one CTA
+// 64 registers: two CTAs per SM, measured 2.7% faster than the compiler's 70 registers
+// and one CTA. ONE_HI: the pair's constants hold for every block of the launch;
+// otherwise they are formed for the high word of each lane's own block index.
+template <bool ONE_HI>
 __global__ void __maxnreg__(64) q4_perturb_kernel(const __grid_constant__ Q4Params p) {
     constexpr int E = kQ4Epl, NB = E / 4, NW = E / 8;
     static_assert(kQ4UnitsPerBlock == 2 && NB == 8, "two 32-element lanes per block");
@@ -122,8 +124,8 @@ __global__ void __maxnreg__(64) q4_perturb_kernel(const __grid_constant__ Q4Para
     const uint32_t lane = threadIdx.x & 31u;
     const uint64_t warp = (static_cast<uint64_t>(blockIdx.x) * kThreadsQ4 + threadIdx.x) >> 5;
     const uint64_t n_warps = (static_cast<uint64_t>(gridDim.x) * kThreadsQ4) >> 5;
-    const SeedConst sc = seed_const(Key{p.seed.k0, p.seed.k1, p.seed.step, p.seed.sample});
-    const float2 eps2 = splat(p.seed.coef);
+    SeedParam sc = seed_param(p.seed, p.block_hi, p.eps);
+    const float2 eps2 = splat(p.eps);
     uint32_t s = 0;
     // all 32 lanes run every iteration (the block maximum is a warp shuffle)
     for (uint64_t wt = warp; wt * 32u < p.n_units; wt += n_warps) {
@@ -162,13 +164,18 @@ __global__ void __maxnreg__(64) q4_perturb_kernel(const __grid_constant__ Q4Para
         // wv[2b] = elements (4b, 4b + 2), wv[2b + 1] = (4b + 1, 4b + 3)
         float2 wv[E / 2];
         const uint64_t blk0 = (g.fo + static_cast<uint64_t>(i0)) >> 2;  // fo % 4 == 0
-        uint4 wcur = philox_block(sc, static_cast<uint32_t>(blk0), static_cast<uint32_t>(blk0 >> 32));
+        const uint32_t blk = static_cast<uint32_t>(blk0);
+        uint4 wcur;
+        if constexpr (!ONE_HI) sc = seed_param(p.seed, static_cast<uint32_t>(blk0 >> 32), p.eps);
+        wcur = philox_block(sc, blk);
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
             uint4 wnext;
-            if (b + 1 < NB)
-                wnext = philox_block(sc, static_cast<uint32_t>(blk0 + b + 1),
-                                     static_cast<uint32_t>((blk0 + b + 1) >> 32));
+            if (b + 1 < NB) {
+                if constexpr (!ONE_HI)
+                    sc = seed_param(p.seed, static_cast<uint32_t>((blk0 + b + 1) >> 32), p.eps);
+                wnext = philox_block(sc, blk + b + 1);
+            }
             const Polar2 o = polar2(wcur);
             if (b + 1 < NB) wcur = wnext;
             const float2 rc = mul2(eps2, o.rr);
@@ -237,7 +244,32 @@ __global__ void __maxnreg__(64) q4_perturb_kernel(const __grid_constant__ Q4Para
     }
 }
 
-std::atomic<int> g_q4_grid[64];
+std::atomic<int> g_q4_grid[2][64];
+
+template <bool ONE_HI>
+cudaError_t launch_q4_t(const Q4Params& p, int grid_ctas, cudaStream_t stream) {
+    int grid = grid_ctas;
+    if (grid <= 0) {
+        int dev = 0;
+        cudaError_t err = cudaGetDevice(&dev);
+        if (err != cudaSuccess) return err;
+        grid = dev < 64 ? g_q4_grid[ONE_HI][dev].load(std::memory_order_relaxed) : 0;
+        if (grid <= 0) {
+            int sms = 0, per_sm = 0;
+            err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            if (err != cudaSuccess) return err;
+            err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, q4_perturb_kernel<ONE_HI>,
+                                                                kThreadsQ4, 0);
+            if (err != cudaSuccess) return err;
+            grid = sms * (per_sm > 0 ? per_sm : 1);
+            if (dev < 64) g_q4_grid[ONE_HI][dev].store(grid, std::memory_order_relaxed);
+        }
+        const uint64_t needed = (p.n_units + kThreadsQ4 - 1) / kThreadsQ4;
+        if (needed < static_cast<uint64_t>(grid)) grid = static_cast<int>(needed);
+    }
+    q4_perturb_kernel<ONE_HI><<<grid, kThreadsQ4, 0, stream>>>(p);
+    return cudaGetLastError();
+}
 
 }  // namespace
 
@@ -247,27 +279,7 @@ void q4_levels_host(float out[16]) {
 
 cudaError_t launch_q4_perturb(const Q4Params& p, int grid_ctas, cudaStream_t stream) {
     if (p.n_units == 0) return cudaSuccess;
-    int grid = grid_ctas;
-    if (grid <= 0) {
-        int dev = 0;
-        cudaError_t err = cudaGetDevice(&dev);
-        if (err != cudaSuccess) return err;
-        grid = dev < 64 ? g_q4_grid[dev].load(std::memory_order_relaxed) : 0;
-        if (grid <= 0) {
-            int sms = 0, per_sm = 0;
-            err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (err != cudaSuccess) return err;
-            err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, q4_perturb_kernel,
-                                                                kThreadsQ4, 0);
-            if (err != cudaSuccess) return err;
-            grid = sms * (per_sm > 0 ? per_sm : 1);
-            if (dev < 64) g_q4_grid[dev].store(grid, std::memory_order_relaxed);
-        }
-        const uint64_t needed = (p.n_units + kThreadsQ4 - 1) / kThreadsQ4;
-        if (needed < static_cast<uint64_t>(grid)) grid = static_cast<int>(needed);
-    }
-    q4_perturb_kernel<<<grid, kThreadsQ4, 0, stream>>>(p);
-    return cudaGetLastError();
+    return p.one_hi ? launch_q4_t<true>(p, grid_ctas, stream) : launch_q4_t<false>(p, grid_ctas, stream);
 }
 
 }  // namespace jb

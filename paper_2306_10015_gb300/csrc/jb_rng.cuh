@@ -38,13 +38,9 @@
 #pragma once
 #include <cstdint>
 
-namespace jb {
+#include "jb_internal.h"
 
-// Philox4x32 round multipliers and key increments (Salmon et al. 2011).
-constexpr uint32_t kPhiloxM0 = 0xD2511F53u;
-constexpr uint32_t kPhiloxM1 = 0xCD9E8D57u;
-constexpr uint32_t kPhiloxW0 = 0x9E3779B9u;
-constexpr uint32_t kPhiloxW1 = 0xBB67AE85u;
+namespace jb {
 
 // Polynomials (fit_poly.py).
 constexpr float kLogP0 = 0x1.5555p+0f, kLogP1 = 0x1.99d29ep-1f, kLogP2 = 0x1.1eb3a2p-1f,
@@ -55,30 +51,6 @@ constexpr float kSinS0 = -0x1.4abbbep-4f, kSinS1 = 0x1.465facp-9f, kSinS2 = -0x1
 constexpr float kCosC0 = -0x1.3bd3ccp-2f, kCosC1 = 0x1.03c1b0p-6f, kCosC2 = -0x1.55b2b6p-12f,
                 kCosC3 = 0x1.d4f7eep-19f;
 constexpr float kTwoLn2 = 0x1.62e430p+0f;
-
-struct Key {
-    uint32_t k0, k1;       // machine id, low and high word
-    uint32_t step, sample; // counter words 2 and 3
-};
-
-// Per-seed constants: the first round's product of counter word 2 (the step)
-// is the same for every block of a seed.
-struct SeedConst {
-    uint32_t k0, k1;
-    uint32_t a_hi, a_lo;  // M1 * step
-    uint32_t c;           // sample ^ k1
-};
-
-__device__ __forceinline__ SeedConst seed_const(const Key& key) {
-    const uint64_t a = static_cast<uint64_t>(kPhiloxM1) * key.step;
-    SeedConst s;
-    s.k0 = key.k0;
-    s.k1 = key.k1;
-    s.a_hi = static_cast<uint32_t>(a >> 32);
-    s.a_lo = static_cast<uint32_t>(a);
-    s.c = key.sample ^ key.k1;
-    return s;
-}
 
 // One Philox round on (x0, x1, x2, x3) with round key (k0, k1).
 __device__ __forceinline__ void philox_round(uint32_t& x0, uint32_t& x1, uint32_t& x2,
@@ -93,43 +65,43 @@ __device__ __forceinline__ void philox_round(uint32_t& x0, uint32_t& x1, uint32_
     x2 = y2;
 }
 
-// The seed-independent part of round 1 for block (b_lo, b_hi): the product of
-// counter word 0 (the block's low word) and its high word. Every seed of an update
-// shares it.
+// The seed-independent part of round 1 for the block with low word b_lo: M0 * b_lo.
+// Every seed of an update shares it.
 struct BlockCtr {
-    uint32_t p_hi, p_lo;  // M0 * b_lo
-    uint32_t b_hi;
+    uint32_t p_hi, p_lo;
 };
 
-__device__ __forceinline__ BlockCtr block_ctr(uint32_t b_lo, uint32_t b_hi) {
+__device__ __forceinline__ BlockCtr block_ctr(uint32_t b_lo) {
     const uint64_t p0 = static_cast<uint64_t>(kPhiloxM0) * b_lo;
     BlockCtr c;
     c.p_hi = static_cast<uint32_t>(p0 >> 32);
     c.p_lo = static_cast<uint32_t>(p0);
-    c.b_hi = b_hi;
     return c;
 }
 
-// Four words of Philox4x32-10 for block c under the seed's constants: round 1 from
-// the per-seed and per-block products, rounds 2 .. 10 in full.
-__device__ __forceinline__ uint4 philox_block(const SeedConst& s, const BlockCtr& c) {
-    uint32_t x0 = s.a_hi ^ c.b_hi ^ s.k0;
-    uint32_t x1 = s.a_lo;
-    uint32_t x2 = c.p_hi ^ s.c;
-    uint32_t x3 = c.p_lo;
+// Four words of Philox4x32-10 for block c under the pair's constants. Round 1 is the
+// block's product and constants of the pair; round 2 needs one product (the other one's
+// factor does not depend on the block's low word, so the host forms it, seed_param);
+// rounds 3 .. 10 in full: 17 wide multiplies.
+__device__ __forceinline__ uint4 philox_block(const SeedParam& s, const BlockCtr& c) {
+    const uint64_t p1 = static_cast<uint64_t>(kPhiloxM1) * (c.p_hi ^ s.c2);
+    uint32_t x0 = static_cast<uint32_t>(p1 >> 32) ^ s.c0;
+    uint32_t x1 = static_cast<uint32_t>(p1);
+    uint32_t x2 = c.p_lo ^ s.n2;
+    uint32_t x3 = s.n3;
     uint32_t k0 = s.k0, k1 = s.k1;
 #pragma unroll
-    for (int r = 1; r < 10; ++r) {
+    for (int r = 2; r < 10; ++r) {
+        philox_round(x0, x1, x2, x3, k0, k1);
         k0 += kPhiloxW0;
         k1 += kPhiloxW1;
-        philox_round(x0, x1, x2, x3, k0, k1);
     }
     return make_uint4(x0, x1, x2, x3);
 }
 
-// Four words of Philox4x32-10 block (b_lo, b_hi).
-__device__ __forceinline__ uint4 philox_block(const SeedConst& s, uint32_t b_lo, uint32_t b_hi) {
-    return philox_block(s, block_ctr(b_lo, b_hi));
+// Four words of the block with low word b_lo.
+__device__ __forceinline__ uint4 philox_block(const SeedParam& s, uint32_t b_lo) {
+    return philox_block(s, block_ctr(b_lo));
 }
 
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -166,8 +138,11 @@ __device__ __forceinline__ float shift_under(uint32_t hi, uint32_t lo, int n) {
     return __uint_as_float(__funnelshift_r(lo, hi, n));
 }
 
+// (bits & keep) | set in one instruction
 __device__ __forceinline__ float masked(uint32_t bits, uint32_t keep, uint32_t set) {
-    return __uint_as_float((bits & keep) | set);
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(r) : "r"(bits), "r"(keep), "r"(set));
+    return __uint_as_float(r);
 }
 
 __device__ __forceinline__ Polar2 polar2(uint4 w) {
@@ -192,9 +167,10 @@ __device__ __forceinline__ Polar2 polar2(uint4 w) {
 
     // ---- angle ----
     const uint32_t tA = w.y + 0x20000000u, tB = w.w + 0x20000000u;
-    // [1, 2) from bits 29 .. 8 and a last bit for the half: 2 (.) - 3 = x, exact
-    const float2 x = fma2(make_float2(masked(tA >> 7, 0x7FFFFEu, 0x3F800001u),
-                                      masked(tB >> 7, 0x7FFFFEu, 0x3F800001u)),
+    // [1, 2) from bits 29 .. 8 and a last bit for the half: 2 (.) - 3 = x, exact. The
+    // bits above become the exponent's low ones.
+    const float2 x = fma2(make_float2(shift_under(0x3F800000u >> 25, tA | 0xC0000080u, 7),
+                                      shift_under(0x3F800000u >> 25, tB | 0xC0000080u, 7)),
                           splat(2.0f), splat(-3.0f));
     const float2 xx = mul2(x, x);
     float2 ps = fma2(xx, splat(kSinS2), splat(kSinS1));
@@ -228,9 +204,9 @@ __device__ __forceinline__ GaussPair box_muller2(uint4 w) {
     return g;
 }
 
-// The four Gaussians of block (b_lo, b_hi), elements 4b .. 4b + 3.
-__device__ __forceinline__ float4 block_gaussians(const SeedConst& s, uint32_t b_lo, uint32_t b_hi) {
-    const GaussPair g = box_muller2(philox_block(s, b_lo, b_hi));
+// The four Gaussians of the block with low word b_lo, elements 4b .. 4b + 3.
+__device__ __forceinline__ float4 block_gaussians(const SeedParam& s, uint32_t b_lo) {
+    const GaussPair g = box_muller2(philox_block(s, b_lo));
     return make_float4(g.even.x, g.odd.x, g.even.y, g.odd.y);
 }
 
