@@ -31,6 +31,8 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cstddef>
+#include <cstring>
 #include <type_traits>
 
 #include "jb_internal.h"
@@ -51,10 +53,17 @@ namespace {
 //                    bf16 2 x 512: 2696 (2 x 768: 2755, 3 x 512: 2782)
 //   one pair         fp32 4 x 1024: 319 (4 x 768: 328, 4 x 512: 329; HBM alone: 316)
 //                    bf16 4 x 1024: 289 (4 x 768: 293, 4 x 512: 302, 8 x 768: 284)
+// Small tables take one vector per thread in every kernel, and their launch fewer
+// parameter bytes: a scheduler needs about one warp's worth of blocks to be busy, so what
+// counts is that all 608 have some. The line lies where the large shape gives most of its
+// 16 warps per SM a tile (K = 32 update, us, one vector / large shape; fp32 512K elements
+// 27 / 29, 1M 43 / 40, 2M 84 / 77; bf16 512K 25 / 33, 1M 43 / 47, 1.5M 62 / 59, 3M 111 / 103).
 template <int V_, int THREADS_, int UNROLL_>
 struct Shape {
     static constexpr int V = V_, THREADS = THREADS_, UNROLL = UNROLL_;
 };
+
+constexpr uint64_t kSmallTiles = 1600;  // tiles of the large shape
 
 template <typename T>
 struct Traits;
@@ -64,6 +73,7 @@ struct Traits<float> {
     using Update = Shape<5, 512, 2>;
     using General = Shape<4, 512, 2>;
     using Pair = Shape<4, 1024, 1>;
+    using Small = Shape<1, 512, 2>;
 };
 template <>
 struct Traits<__nv_bfloat16> {
@@ -71,6 +81,7 @@ struct Traits<__nv_bfloat16> {
     using Update = Shape<3, 512, 2>;
     using General = Shape<2, 512, 2>;
     using Pair = Shape<4, 1024, 1>;
+    using Small = Shape<1, 512, 2>;
 };
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
@@ -624,37 +635,42 @@ cudaError_t persistent_grid(K kernel, int threads, GridCache& cache, int* grid) 
     return cudaSuccess;
 }
 
-// Launches `kernel` on the packed table.
-template <typename P, typename K>
-cudaError_t launch(K kernel, int threads, GridCache& cache, P& p, int grid_ctas, cudaStream_t stream) {
+// Launches `kernel` on the packed table. A warp takes spans of up to four tiles, so that
+// the lookup of their segment is paid once; fewer where a warp would get less than eight
+// spans, so that all warps end at about the same time.
+template <typename S, typename P, typename K>
+cudaError_t launch(K kernel, GridCache& cache, P& p, int grid_ctas, cudaStream_t stream) {
     int grid = grid_ctas;
     if (grid <= 0) {
-        cudaError_t err = persistent_grid(kernel, threads, cache, &grid);
+        cudaError_t err = persistent_grid(kernel, S::THREADS, cache, &grid);
         if (err != cudaSuccess) return err;
-        const uint32_t needed = (p.n_tiles + p.span - 1) / p.span;
-        if (needed < static_cast<uint32_t>(grid)) grid = static_cast<int>(needed);
     }
-    kernel<<<grid, threads, 0, stream>>>(p);
+    const uint64_t warps = static_cast<uint64_t>(grid) * (S::THREADS / 32);
+    p.span = 4;
+    while (p.span > 1 && p.n_tiles < 8 * warps * p.span) p.span /= 2;
+    const uint32_t needed = (p.n_tiles + p.span - 1) / p.span;
+    if (grid_ctas <= 0 && needed < static_cast<uint32_t>(grid)) grid = static_cast<int>(needed);
+    kernel<<<grid, S::THREADS, 0, stream>>>(p);
     return cudaGetLastError();
 }
 
-template <typename T, typename P>
+template <typename T, bool SMALL, typename P>
 cudaError_t launch_work(const Job& job, P& p) {
     static GridCache caches[3];
-    using U = typename Traits<T>::Update;
-    using G = typename Traits<T>::General;
-    using S = typename Traits<T>::Pair;
+    using U = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::Update>;
+    using G = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::General>;
+    using S = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::Pair>;
     const int ctas = job.grid_ctas;
     if constexpr (std::is_same<typename P::Seg, SegParamOut>::value) {
         if (p.n_seeds == 1)
-            return launch(one_seed_kernel<T, S, kAddToDst, P>, S::THREADS, caches[0], p, ctas, job.stream);
-        return launch(general_update_kernel<T, G, P>, G::THREADS, caches[1], p, ctas, job.stream);
+            return launch<S>(one_seed_kernel<T, S, kAddToDst, P>, caches[0], p, ctas, job.stream);
+        return launch<G>(general_update_kernel<T, G, P>, caches[1], p, ctas, job.stream);
     } else {
         if (job.work == kPerturb)
-            return launch(one_seed_kernel<T, S, kPerturbInPlace, P>, S::THREADS, caches[0], p, ctas, job.stream);
+            return launch<S>(one_seed_kernel<T, S, kPerturbInPlace, P>, caches[0], p, ctas, job.stream);
         if (p.n_seeds == 1)
-            return launch(one_seed_kernel<T, S, kAddInPlace, P>, S::THREADS, caches[1], p, ctas, job.stream);
-        return launch(seeded_kernel<T, U, P>, U::THREADS, caches[2], p, ctas, job.stream);
+            return launch<S>(one_seed_kernel<T, S, kAddInPlace, P>, caches[1], p, ctas, job.stream);
+        return launch<U>(seeded_kernel<T, U, P>, caches[2], p, ctas, job.stream);
     }
 }
 
@@ -664,9 +680,13 @@ template <typename T, typename SEG>
 cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size_t n_segs) {
     using P = Launch<SEG, kParamBytes>;
     constexpr uint64_t E = Traits<T>::E, ES = sizeof(T);
-    const uint64_t tile_vec = 32ull * (job.n_seeds == 1        ? Traits<T>::Pair::V
-                                       : job.work == kGeneral ? Traits<T>::General::V
-                                                              : Traits<T>::Update::V);
+    const uint64_t big_vec = 32ull * (job.n_seeds == 1        ? Traits<T>::Pair::V
+                                      : job.work == kGeneral ? Traits<T>::General::V
+                                                             : Traits<T>::Update::V);
+    uint64_t big_tiles = 0;
+    for (size_t k = 0; k < n_segs; ++k) big_tiles += (segs[k].n + E * big_vec - 1) / (E * big_vec);
+    const bool small = big_tiles < kSmallTiles;
+    const uint64_t tile_vec = small ? 32u : big_vec;
     static thread_local P p;  // ~32 KB: keep it off the stack
     p.n_seeds = static_cast<uint32_t>(job.n_seeds);
     p.write_src = job.write_src ? 1u : 0u;
@@ -710,11 +730,20 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
         table[count].tile0 = static_cast<uint32_t>(tiles);
         p.n_segs = static_cast<uint32_t>(count);
         p.n_tiles = static_cast<uint32_t>(tiles);
-        p.span = 4;
         SeedParam* sp = reinterpret_cast<SeedParam*>(p.data);
         for (int k = 0; k < job.n_seeds; ++k) sp[k] = seed_param(job.seeds[k], hi, job.coef[k]);
         for (int k = 0; k < job.n_groups; ++k) sp[job.group_end[k] - 1].ends_group = 1u;
-        const cudaError_t err = launch_work<T>(job, p);
+        cudaError_t err;
+        const size_t used = p.seg_at + (count + 1) * sizeof(SEG);
+        if (!small) {
+            err = launch_work<T, false>(job, p);
+        } else if (used > kSmallParamBytes) {
+            err = launch_work<T, true>(job, p);
+        } else {
+            Launch<SEG, kSmallParamBytes> q;
+            std::memcpy(&q, &p, offsetof(P, data) + used);
+            err = launch_work<T, true>(job, q);
+        }
         if (err != cudaSuccess) return err;
     }
     return cudaSuccess;

@@ -1,0 +1,121 @@
+"""The kernel shapes chosen by table size, and segments cut where the high word of the
+Philox block index changes: the result does not depend on either.
+
+A table that takes the large shape must give, bit for bit, what small tables over its
+pieces give (they take the one-vector shape); those are checked against the oracle in
+test_gpu_parity.py and, for the cuts, here."""
+import numpy as np
+import pytest
+
+import oracle
+import synthetic
+from jbtest_util import check_theta, to_device, to_host, update_scale
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+F32 = np.float32
+LR, DENOM, QS = float(F32(1e-3)), 3.0, 16.0
+
+
+@pytest.fixture(scope="module")
+def jb():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2306_10015_gb300 import build
+    build.build()
+    import paper_2306_10015_gb300 as pkg
+    pkg.lib()
+    return pkg
+
+
+def pairs(K):
+    seeds = [(int(m), 5, i % 3) for i, m in enumerate(synthetic.machine_ids(K, 61))]
+    return seeds, synthetic.byte_codes(K, 61)
+
+
+def operations(jb):
+    def replay(t):
+        (s1, q1), (s2, q2) = pairs(1), pairs(3)
+        jb.jb_replay_updates(t, [(s1, q1, LR, DENOM), (s2, q2, LR, DENOM), (s1, q1, LR, 1.0)], QS)
+
+    def into(t, K):
+        out = [torch.zeros_like(x) for x in t.tensors]
+        jb.jb_apply_updates_from(t, jb.ParamTable(out, t.flat_offsets), *pairs(K), LR, DENOM, QS)
+        for x, o in zip(t.tensors, out):
+            x.copy_(o)
+
+    return {"perturb": lambda t: jb.jb_perturb(t, (7, 8, 9), 1e-3),
+            "update K=1": lambda t: jb.jb_apply_updates(t, *pairs(1), LR, DENOM, QS),
+            "update K=2": lambda t: jb.jb_apply_updates(t, *pairs(2), LR, DENOM, QS),
+            "update K=5": lambda t: jb.jb_apply_updates(t, *pairs(5), LR, DENOM, QS),
+            "from K=1": lambda t: into(t, 1), "from K=4": lambda t: into(t, 4), "replay": replay}
+
+
+# elements of a warp tile of the large shapes: update, replay, one pair
+TILES = {torch.float32: (640, 512, 512), torch.bfloat16: (768, 512, 1024)}
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("tiles,extra,shift", [(1599, 0, 0), (1600, -1, 0), (1600, 1, 0), (1700, 5, 3),
+                                               (1700, 31 * 8, 0)])
+def test_large_shape_equals_small_pieces(jb, dtype, tiles, extra, shift):
+    for name, op in operations(jb).items():
+        t = TILES[dtype][0 if name.startswith("update") and name[-1] != "1" else
+                         (2 if name[-1] == "1" or name == "perturb" else 1)]
+        n = tiles * t + extra
+        torch.manual_seed(n)
+        base = torch.randn(n + 16, device="cuda").mul_(0.02).to(dtype)
+        whole, parts = base.clone(), base.clone()
+        op(jb.ParamTable([whole[shift:shift + n]], [11]))
+        cuts = [0, 1, 9, 4099] + list(range(300_001, n, 300_001)) + [n - 3, n]
+        for a, b in zip(cuts, cuts[1:]):
+            op(jb.ParamTable([parts[shift + a:shift + b]], [11 + a]))
+        torch.cuda.synchronize()
+        assert torch.equal(whole.view(torch.uint8), parts.view(torch.uint8)), name
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("boundary", [1 << 33, 1 << 34, 3 << 33])
+def test_segment_across_a_cut(jb, dtype, boundary):
+    """A segment that crosses a multiple of 2^33 elements (2^34: another high word)."""
+    for before, K in ((1001, 3), (1, 1), (4096, 2)):
+        v = synthetic.normal_values(5003, 0.02, 62)
+        v = v if dtype == "f32" else oracle.round_bf16(v.astype(np.float64))
+        fo = boundary - before
+        dev = to_device(v)
+        seeds, q = pairs(K)
+        jb.jb_apply_updates(jb.ParamTable([dev], [fo]), seeds, q, LR, DENOM, QS)
+        torch.cuda.synchronize()
+        scale = update_scale(v, np.arange(fo, fo + v.size, dtype=np.uint64), seeds, q, LR, DENOM, QS)
+        check_theta(to_host(dev), oracle.update(v, fo, seeds, q, LR, DENOM, QS), scale, f"{boundary}")
+
+
+def test_q4_across_a_high_word(jb):
+    """4-bit tensors whose Philox block indices cross 2^32, or lie above it."""
+    n = 64 * 40 + 33
+    for fos in ([(1 << 34) - 1028], [1 << 34], [64, (1 << 35) + 8]):
+        host, dev = [], []
+        for i, _ in enumerate(fos):
+            codes, scale = oracle.q4_quantize(synthetic.normal_values(n, 0.02, 63 + i).astype(np.float64))
+            host.append((codes, scale))
+            pad = np.zeros(codes.size + 16, dtype=np.uint8)
+            pad[:codes.size] = codes
+            dev.append((torch.from_numpy(pad).cuda(), torch.from_numpy(scale.copy()).cuda(), n))
+        jb.jb_perturb_q4(jb.Q4Table(dev, fos), (3, 4, 5), 1e-3)
+        torch.cuda.synchronize()
+        level = jb.jb_q4_levels().astype(np.float64)
+        for (codes, scale), (dc, ds, _), fo in zip(host, dev, fos):
+            old = np.empty(2 * codes.size, dtype=np.int64)
+            old[0::2], old[1::2] = codes & 15, codes >> 4
+            w = level[old[:n]] * np.repeat(scale, 64)[:n].astype(np.float64)
+            w += float(F32(1e-3)) * oracle.gaussian_range((3, 4, 5), fo, n)
+            want = np.abs(np.pad(w, (0, 64 * scale.size - n))).reshape(-1, 64).max(1)
+            # w' is one fp32 multiply-add of values below 0.2 with z to 1e-6
+            assert np.all(np.abs(ds.cpu().numpy() - want) <= 2e-8 + 1e-9)
+            new = dc.cpu().numpy()[:codes.size].astype(np.int64)
+            got = np.empty(2 * codes.size, dtype=np.int64)
+            got[0::2], got[1::2] = new & 15, new >> 4
+            near = np.abs((w / np.repeat(want, 64)[:n])[:, None] - level[None, :]).argmin(1)
+            # ties within fp32 error of a midpoint: none expected among 2593 weights
+            assert np.count_nonzero(got[:n] != near) <= 1
