@@ -41,7 +41,6 @@ int guarded(F&& body) noexcept {
         return JB_ERR_INVALID_ARG;
     }
 }
-int elems_per_vec(int dtype) { return dtype == JB_F32 ? 4 : 8; }
 
 // Checks the segment table; drops empty segments. Overlap in memory or in
 // global index is an argument error.
@@ -69,30 +68,6 @@ int collect_segments(const jb_segment* segs, int n_segs, int dtype, std::vector<
     for (size_t i = 1; i < by_ptr.size(); ++i)
         if (by_ptr[i - 1].ptr + by_ptr[i - 1].n * es > by_ptr[i].ptr) return JB_ERR_INVALID_ARG;
     return JB_OK;
-}
-
-// Fills params with segments [first, first + count).
-void pack_segments(const std::vector<Seg>& segs, size_t first, size_t count, int dtype,
-                   jb::SumParams& params) {
-    const uint64_t E = static_cast<uint64_t>(elems_per_vec(dtype));
-    const uint64_t es = elem_size(dtype);
-    uint64_t vec = 0;
-    for (size_t i = 0; i < count; ++i) {
-        const Seg& s = segs[first + i];
-        jb::SumSegParam& g = params.segs[i];
-        const uint64_t v_begin = s.fo / E;
-        const uint64_t v_end = (s.fo + s.n + E - 1) / E;
-        // 16-byte vectors of the segment line up with element groups whose global
-        // index is a multiple of E iff ptr - fo * sizeof(T) is 16-byte aligned.
-        const bool aligned = ((s.ptr - s.fo * es) & 15ull) == 0;
-        g.ptr = s.ptr | (aligned ? 1ull : 0ull);
-        g.fo = s.fo;
-        g.n = s.n;
-        g.vec0 = vec;
-        vec += v_end - v_begin;
-    }
-    params.n_segs = static_cast<uint32_t>(count);
-    params.n_vec = vec;
 }
 
 jb::SeedRaw seed_raw(const jb_seed& s) {
@@ -135,7 +110,7 @@ int perturb_impl(const jb_segment* segs, int n_segs, int dtype, jb_seed seed, fl
     if (!std::isfinite(eps)) return JB_ERR_INVALID_ARG;
     if (v.empty()) return JB_OK;
     const jb::SeedRaw raw = seed_raw(seed);
-    jb::Job job{jb::kPerturb, dtype, &raw, &eps, 1, nullptr, 0, false, grid_ctas, stream};
+    jb::Job job{jb::kPerturb, dtype, &raw, &eps, 1, nullptr, 0, false, grid_ctas, stream, nullptr};
     return cuda_status(jb::enqueue(job, v.data(), nullptr, v.size()));
 }
 
@@ -171,7 +146,7 @@ int update_impl(const jb_segment* segs, int n_segs, int dtype, const jb_seed* se
         raw[k] = seed_raw(seeds[i]);
     }
     if (v.empty()) return JB_OK;
-    jb::Job job{jb::kUpdate, dtype, raw.data(), coef.data(), K, nullptr, 0, false, grid_ctas, stream};
+    jb::Job job{jb::kUpdate, dtype, raw.data(), coef.data(), K, nullptr, 0, false, grid_ctas, stream, nullptr};
     return cuda_status(jb::enqueue(job, v.data(), nullptr, v.size()));
 }
 
@@ -286,7 +261,7 @@ int general_impl(const jb_segment* segs, const jb_segment* dsts, int n_segs, int
         const bool last = g1 >= sizes.size();
         // write_src comes with one group only (jb_apply_updates_from): one launch round
         jb::Job job{jb::kGeneral, dtype, raw.data() + s0, coef.data() + s0, static_cast<int>(n),
-                    ends.data(), static_cast<int>(ends.size()), write_src && last, grid_ctas, stream};
+                    ends.data(), static_cast<int>(ends.size()), write_src && last, grid_ctas, stream, nullptr};
         rc = cuda_status(jb::enqueue(job, from.data(), dptr.data(), from.size()));
         if (rc != JB_OK) return rc;
         for (size_t i = 0; i < from.size(); ++i) from[i].ptr = dptr[i];
@@ -352,17 +327,10 @@ int checksum_impl(const jb_segment* segs, int n_segs, int dtype, uint64_t* d_out
     if (rc != JB_OK) return rc;
     if (d_out == nullptr) return JB_ERR_INVALID_ARG;
     if (reinterpret_cast<uint64_t>(d_out) & 7ull) return JB_ERR_MISALIGNED;
-    rc = cuda_status(cudaMemsetAsync(d_out, 0, sizeof(uint64_t), stream));
-    if (rc != JB_OK) return rc;
-    static thread_local jb::SumParams params;  // ~32 KB: keep it off the stack
-    for (size_t first = 0; first < v.size(); first += jb::kMaxSegsSum) {
-        const size_t count = std::min<size_t>(jb::kMaxSegsSum, v.size() - first);
-        pack_segments(v, first, count, dtype, params);
-        rc = cuda_status(jb::launch_checksum(params, dtype, reinterpret_cast<unsigned long long*>(d_out),
-                                             grid_ctas, stream));
-        if (rc != JB_OK) return rc;
-    }
-    return JB_OK;
+    if (v.empty()) return cuda_status(cudaMemsetAsync(d_out, 0, sizeof(uint64_t), stream));
+    jb::Job job{jb::kChecksum, dtype, nullptr, nullptr, 0, nullptr, 0, false, grid_ctas, stream,
+                reinterpret_cast<unsigned long long*>(d_out)};
+    return cuda_status(jb::enqueue(job, v.data(), nullptr, v.size()));
 }
 }  // namespace
 

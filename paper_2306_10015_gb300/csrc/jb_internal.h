@@ -25,7 +25,7 @@
 
 namespace jb {
 
-constexpr int kThreads = 512;  // threads per CTA of the checksum and the generator alone
+constexpr int kThreads = 512;  // threads per CTA of the generator alone
 constexpr int kMaxSeedsPerLaunch = 512;
 constexpr int kMaxGroupsPerLaunch = 512;
 constexpr uint64_t kPieceElems = 1ull << 33;  // segments are cut at multiples of this index
@@ -72,7 +72,7 @@ __host__ __device__ inline SeedParam seed_param(const SeedRaw& s, uint32_t block
 struct SegParam {
     uint64_t base;   // device address of the segment's first window (its element `head` is element 0)
     uint64_t end;    // elements of the segment are [head, end) of its windows
-    uint32_t blk0;   // low word of the Philox block index of the first window
+    uint32_t blk0;   // low word of the Philox block index of the first window (checksum: its own)
     uint32_t tile0;  // first tile
     uint32_t head;   // elements of the first window before the segment (0 .. E - 1)
     uint32_t full;   // vectors [head ? 1 : 0, full) take 16-byte accesses; 0: none does
@@ -90,7 +90,8 @@ struct Launch {
     uint32_t n_segs;
     uint32_t n_tiles;
     uint32_t span;       // consecutive tiles that a warp takes at a time
-    uint32_t write_src;  // write the result to the source too
+    uint32_t write_src;  // write the result to the source too; checksum: one CTA, store the sum
+    uint32_t window_hi;  // checksum: high word of every window index
     uint32_t seg_at;     // byte offset of the segment table in `data`; the pairs are at 0
     alignas(16) unsigned char data[BYTES];
 };
@@ -105,24 +106,6 @@ static_assert(sizeof(Launch<SegParam, kParamBytes>) <= 32764, "launch exceeds th
 struct Seg {
     uint64_t ptr, fo, n;
 };
-
-// Checksum: no pairs, and windows keep their 64-bit index.
-constexpr int kMaxSegsSum = 1000;
-
-struct SumSegParam {
-    uint64_t ptr;   // device address; bit 0 set when the 16-byte vector path applies
-    uint64_t fo;    // global index of element 0
-    uint64_t n;     // elements
-    uint64_t vec0;  // first launch vector of this segment
-};
-
-struct SumParams {
-    uint32_t n_segs;
-    uint64_t n_vec;  // vectors in this launch
-    SumSegParam segs[kMaxSegsSum];
-};
-
-static_assert(sizeof(SumParams) <= 32764, "checksum launch exceeds the parameter space");
 
 // 4-bit weights: codes (two per byte, element 2i in the low nibble) and one fp32
 // scale per 64 elements. A segment owns units [unit0, unit0 + units), kQ4UnitsPerBlock
@@ -156,8 +139,9 @@ enum DType { kF32 = 0, kBF16 = 1 };
 
 // What a launch runs: PerturbParameters (one pair, theta + eps z as one fused
 // multiply-add), the in-place update, or the general update (source to destination,
-// groups). One pair in one group takes the one-pair kernel in both updates.
-enum Work { kPerturb = 0, kUpdate = 1, kGeneral = 2 };
+// groups). One pair in one group takes the one-pair kernel in both updates. The checksum
+// has no pairs.
+enum Work { kPerturb = 0, kUpdate = 1, kGeneral = 2, kChecksum = 3 };
 
 struct Job {
     Work work;
@@ -170,14 +154,13 @@ struct Job {
     bool write_src;
     int grid_ctas;  // <= 0: the persistent grid
     cudaStream_t stream;
+    unsigned long long* sum;  // checksum: device address of the result
 };
 
 // Packs the segments into launches of the job and enqueues them. dst: the general
 // update's destinations, one per segment (n_segs > 0).
 cudaError_t enqueue(const Job& job, const Seg* segs, const uint64_t* dst, size_t n_segs);
 
-cudaError_t launch_checksum(const SumParams& p, int dtype, unsigned long long* out, int grid_ctas,
-                            cudaStream_t s);
 cudaError_t launch_debug_philox(SeedRaw seed, uint64_t first_block, uint64_t n_blocks,
                                 uint32_t* out, cudaStream_t s);
 cudaError_t launch_debug_philox_fold(SeedRaw seed, uint64_t first_block, uint64_t n_blocks,

@@ -51,6 +51,8 @@ namespace {
 //                    bf16 3 x 512: 4099 (2 x 512: 4267, 2 x 768: 4157, 2 x 640: 4176)
 //   replay, 10 pairs fp32 4 x 512: 2655 (4 x 768: 2777, 6 x 512: 2766)
 //                    bf16 2 x 512: 2696 (2 x 768: 2755, 3 x 512: 2782)
+//   checksum         fp32 6 x 512: 152.0 (8 x 512: 153.4, 4 x 512: 157), bf16 79.9 (81.1, 83.2);
+//                    1.3B bf16 359 either way: 7.3 TB/s
 //   one pair         fp32 4 x 1024: 319 (4 x 768: 328, 4 x 512: 329; HBM alone: 316)
 //                    bf16 4 x 1024: 289 (4 x 768: 293, 4 x 512: 302, 8 x 768: 284)
 // Small tables take one vector per thread in every kernel, and their launch fewer
@@ -73,6 +75,7 @@ struct Traits<float> {
     using Update = Shape<5, 512, 2>;
     using General = Shape<4, 512, 2>;
     using Pair = Shape<4, 1024, 1>;
+    using Sum = Shape<6, 512, 1>;
     using Small = Shape<1, 512, 2>;
 };
 template <>
@@ -81,6 +84,7 @@ struct Traits<__nv_bfloat16> {
     using Update = Shape<3, 512, 2>;
     using General = Shape<2, 512, 2>;
     using Pair = Shape<4, 1024, 1>;
+    using Sum = Shape<6, 512, 1>;
     using Small = Shape<1, 512, 2>;
 };
 
@@ -167,19 +171,23 @@ __device__ __forceinline__ uint32_t find_seg(const P& p, uint32_t s, uint32_t t)
 __device__ __forceinline__ uint64_t dst_of(const SegParam& g) { return g.base; }
 __device__ __forceinline__ uint64_t dst_of(const SegParamOut& g) { return g.dst; }
 
-// Runs op(x, blk) on each of this warp's tiles and stores the result (to the
-// destination table when TO_DST, and then also back to the source when also_src): x[j]
-// is vector 32 j + lane of the tile in storage form, blk the low word of the first
-// Philox block of x[0] (x[j] is at blk + 32 j B). A warp takes spans of p.span
+enum Store { kInPlace, kToDst, kNowhere };
+
+// Runs op(x, blk, present) on each of this warp's tiles and stores the result (in place,
+// to the destination table, and then also back to the source when also_src, or nowhere):
+// x[j] is vector 32 j + lane of the tile in storage form, blk the low word of the first
+// Philox block of x[0] (x[j] is at blk + 32 j B; stored nowhere: of the window, and B is
+// 1), and present (stored nowhere only) how many vectors the segment has from x[0] on. A
+// warp takes spans of p.span
 // consecutive tiles, strided by the number of warps in the grid; tiles that follow one
 // another go to different SMs, so that a few tiles occupy as many SMs. Which warp
 // handles a tile never changes a result: every element's value depends only on its own
 // stored value, its global index and the seeds. Vectors that are partial (the ends of a
 // segment), or whose segment lies off the 16-byte grid, go element by element.
-template <typename T, typename S, bool TO_DST, typename P, typename Op>
+template <typename T, typename S, Store TO, typename P, typename Op>
 __device__ __forceinline__ void visit_tiles(const P& p, bool also_src, Op&& op) {
     constexpr int E = Traits<T>::E, V = S::V;
-    constexpr uint32_t B = E / 4, kTileVec = 32u * V;
+    constexpr uint32_t B = TO == kNowhere ? 1 : E / 4, kTileVec = 32u * V;
     const uint32_t lane = threadIdx.x & 31u;
     const uint64_t span = p.span;
     const uint64_t stride = span * (static_cast<uint64_t>(gridDim.x) * (S::THREADS / 32));
@@ -218,9 +226,16 @@ __device__ __forceinline__ void visit_tiles(const P& p, bool also_src, Op&& op) 
                         }
                     }
                 }
-                op(x, blk);
+                if constexpr (TO == kNowhere) {
+                    const uint64_t vecs = (g.end + E - 1) / E;  // a tile has at least one
+                    op(x, blk, fast ? kTileVec : static_cast<uint32_t>(vecs < v + lane ? 0 : vecs - v - lane));
+                } else {
+                    op(x, blk);
+                }
+                constexpr bool TO_DST = TO == kToDst;
                 const uint64_t out = TO_DST ? dst : src;
-                if (fast) {
+                if constexpr (TO == kNowhere) {
+                } else if (fast) {
 #pragma unroll
                     for (int j = 0; j < V; ++j) {
                         store_vec(out + 512ull * j, x[j]);
@@ -328,7 +343,7 @@ __device__ __forceinline__ void update_tile(const P& p, uint4 (&x)[S::V], uint32
 
 template <typename T, typename S, typename P>
 __global__ void __launch_bounds__(S::THREADS) seeded_kernel(const __grid_constant__ P p) {
-    visit_tiles<T, S, false>(p, false, [&](uint4 (&x)[S::V], uint32_t blk) {
+    visit_tiles<T, S, kInPlace>(p, false, [&](uint4 (&x)[S::V], uint32_t blk) {
         update_tile<T, S, false>(p, x, blk);
     });
 }
@@ -373,7 +388,7 @@ enum OneSeed { kPerturbInPlace = 0, kAddInPlace = 1, kAddToDst = 2 };
 template <typename T, typename S, int MODE, typename P>
 __global__ void __launch_bounds__(S::THREADS) one_seed_kernel(const __grid_constant__ P p) {
     constexpr bool TO_DST = MODE == kAddToDst;
-    visit_tiles<T, S, TO_DST>(p, TO_DST && p.write_src != 0u, [&](uint4 (&x)[S::V], uint32_t blk) {
+    visit_tiles<T, S, TO_DST ? kToDst : kInPlace>(p, TO_DST && p.write_src != 0u, [&](uint4 (&x)[S::V], uint32_t blk) {
         one_seed_tile<T, S::V, MODE == kPerturbInPlace>(p, x, blk);
     });
 }
@@ -383,7 +398,7 @@ __global__ void __launch_bounds__(S::THREADS) one_seed_kernel(const __grid_const
 // group, exactly as successive in-place updates would round.
 template <typename T, typename S, typename P>
 __global__ void __launch_bounds__(S::THREADS) general_update_kernel(const __grid_constant__ P p) {
-    visit_tiles<T, S, true>(p, p.write_src != 0u, [&](uint4 (&x)[S::V], uint32_t blk) {
+    visit_tiles<T, S, kToDst>(p, p.write_src != 0u, [&](uint4 (&x)[S::V], uint32_t blk) {
         update_tile<T, S, true>(p, x, blk);
     });
 }
@@ -393,17 +408,11 @@ __global__ void __launch_bounds__(S::THREADS) general_update_kernel(const __grid
 // storage words (elements outside the segment read as 0) keyed by the window
 // index; per window (x1:x0) + (x3:x2). Integer addition is order-free, so one
 // atomic add per CTA gives the same bits for any grid. Bound by HBM: one read
-// of theta, one wide multiply pair per window and round.
+// of theta, one wide multiply pair per window and round. The tiles are those of the
+// updates (1200 tensors of 20M elements in all: 111 -> 41 us against tiles that may cross
+// tensors and a linear search for the tensor).
 constexpr uint32_t kSumKey0 = 0x6A09E667u, kSumKey1 = 0xF3BCC908u;
 constexpr int kSumRounds = 4;
-#ifndef JB_SUM_V
-#define JB_SUM_V 8
-#endif
-constexpr int kSumV = JB_SUM_V;  // 16-byte loads in flight per thread
-#ifndef JB_SUM_S
-#define JB_SUM_S 4
-#endif
-constexpr int kSumS = JB_SUM_S;  // warp tiles per span
 
 __device__ __forceinline__ uint64_t window_hash(uint64_t win, uint4 w) {
     uint32_t x0 = w.x, x1 = w.y, x2 = w.z, x3 = w.w;
@@ -420,131 +429,31 @@ __device__ __forceinline__ uint64_t window_hash(uint64_t win, uint4 w) {
     return ((static_cast<uint64_t>(x1) << 32) | x0) + ((static_cast<uint64_t>(x3) << 32) | x2);
 }
 
-// Checksum: the segment table by launch vector.
-struct SumTile {
-    bool fast;       // inside one segment, every vector full and on the 16-byte path
-    uint32_t count;  // vectors in the tile
-    uint64_t base;   // address of the tile's first vector
-    uint64_t win0;   // global window (E-element group) of the first vector
-};
-
-template <int E, int V, int ES>
-__device__ __forceinline__ SumTile sum_tile(const SumParams& p, uint64_t wt, uint32_t& s) {
-    const uint64_t v0 = wt * (32u * V);
-    const uint64_t n_vec = p.n_vec;
-    while (s + 1 < p.n_segs && p.segs[s + 1].vec0 <= v0) ++s;
-    const SumSegParam& g = p.segs[s];
-    const uint64_t seg_end = s + 1 < p.n_segs ? p.segs[s + 1].vec0 : n_vec;
-    const uint64_t vend = v0 + 32u * V < n_vec ? v0 + 32u * V : n_vec;
-    SumTile f;
-    f.win0 = g.fo / E + (v0 - g.vec0);
-    const int64_t i_first = static_cast<int64_t>(f.win0 * E) - static_cast<int64_t>(g.fo);
-    const int64_t i_end = i_first + static_cast<int64_t>(vend - v0) * E;
-    f.fast = vend <= seg_end && (g.ptr & 1ull) && i_first >= 0 && i_end <= static_cast<int64_t>(g.n);
-    f.count = static_cast<uint32_t>(vend - v0);
-    f.base = (g.ptr & ~1ull) + static_cast<uint64_t>(i_first) * ES;
-    return f;
-}
-
-__device__ __forceinline__ uint32_t raw_bits(const float* p) { return __float_as_uint(*p); }
-__device__ __forceinline__ uint32_t raw_bits(const __nv_bfloat16* p) {
-    return *reinterpret_cast<const uint16_t*>(p);
-}
-
-// Checksum terms of warp tile wt on the per-vector path (tiles that cross a
-// segment boundary or lie in a segment off the 16-byte grid): windows are read
-// element by element where they are partial, with elements outside the segment
-// taken as zero bits.
-template <typename T, int V>
-__device__ __forceinline__ uint64_t sum_tile_general(const SumParams& p, uint64_t wt, uint32_t lane,
-                                                     uint32_t& s) {
-    constexpr int E = Traits<T>::E;
-    constexpr int BITS = 8 * static_cast<int>(sizeof(T));
-    const uint64_t n_vec = p.n_vec;
-    const uint32_t n_segs = p.n_segs;
+// blk0 of the segments is the low word of the index of the first window, p.window_hi
+// the high word of all. One CTA alone stores its sum, which saves the clearing of *out.
+template <typename T, typename S, typename P>
+__global__ void __launch_bounds__(S::THREADS) checksum_kernel(const __grid_constant__ P p,
+                                                             unsigned long long* out) {
     uint64_t sum = 0;
+    visit_tiles<T, S, kNowhere>(p, false, [&](uint4 (&x)[S::V], uint32_t win, uint32_t present) {
 #pragma unroll
-    for (int j = 0; j < V; ++j) {
-        const uint64_t vi = wt * (32u * V) + 32u * j + lane;
-        const bool valid = vi < n_vec;
-        if (valid)
-            while (s + 1 < n_segs && p.segs[s + 1].vec0 <= vi) ++s;
-        const SumSegParam& g = p.segs[s];
-        const uint64_t win = g.fo / E + (vi - g.vec0);
-        const int64_t i0 = static_cast<int64_t>(win * E) - static_cast<int64_t>(g.fo);
-        const int64_t n = static_cast<int64_t>(g.n);
-        const T* base = reinterpret_cast<const T*>(g.ptr & ~1ull);
-        uint4 w;
-        if (valid && (g.ptr & 1ull) && i0 >= 0 && i0 + E <= n) {
-            w = __ldcs(reinterpret_cast<const uint4*>(base + i0));
-        } else {
-            uint32_t ww[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-            for (int t = 0; t < E; ++t) {
-                const int64_t i = i0 + t;
-                if (valid && i >= 0 && i < n) ww[t * BITS / 32] |= raw_bits(base + i) << ((t * BITS) % 32);
-            }
-            w = make_uint4(ww[0], ww[1], ww[2], ww[3]);
+        for (int j = 0; j < S::V; ++j) {
+            const uint64_t w = (static_cast<uint64_t>(p.window_hi) << 32) | (win + 32u * j);
+            if (32u * j < present) sum += window_hash(w, x[j]);
         }
-        if (valid) sum += window_hash(win, w);
-    }
-    return sum;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kThreads) checksum_kernel(const __grid_constant__ SumParams p,
-                                                           unsigned long long* out) {
-    constexpr int E = Traits<T>::E;
-    constexpr int V = kSumV;
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint64_t warp = (static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x) >> 5;
-    const uint64_t n_warps = (static_cast<uint64_t>(gridDim.x) * kThreads) >> 5;
-    const uint64_t n_vec = p.n_vec;
-    constexpr int S = kSumS;
-    constexpr uint32_t kTileVec = 32u * V;
-    uint32_t s = 0;
-    uint64_t sum = 0;
-    for (uint64_t ws = warp; ws * (kTileVec * S) < n_vec; ws += n_warps) {
-        const SumTile fs = sum_tile<E, V * S, sizeof(T)>(p, ws, s);
-        if (fs.fast) {
-#pragma unroll 1
-            for (uint32_t done = 0; done < fs.count; done += kTileVec) {
-                const uint64_t base = fs.base + 16ull * done;
-                uint4 w[V];
-                uint64_t win[V];
-                bool valid[V];
-#pragma unroll
-                for (int j = 0; j < V; ++j) {
-                    const uint32_t v = 32u * j + lane;
-                    valid[j] = done + v < fs.count;
-                    win[j] = fs.win0 + done + v;
-                    w[j] = valid[j] ? __ldcs(reinterpret_cast<const uint4*>(base + 16ull * v))
-                                    : make_uint4(0u, 0u, 0u, 0u);
-                }
-#pragma unroll
-                for (int j = 0; j < V; ++j)
-                    if (valid[j]) sum += window_hash(win[j], w[j]);
-            }
-            continue;
-        }
-#pragma unroll 1
-        for (int u = 0; u < S; ++u) {
-            const uint64_t wt = ws * S + u;
-            if (wt * kTileVec >= n_vec) break;
-            sum += sum_tile_general<T, V>(p, wt, lane, s);
-        }
-    }
+    });
     // CTA reduction; every thread reaches the barrier
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) sum += __shfl_down_sync(0xFFFFFFFFu, sum, d);
-    __shared__ uint64_t part[kThreads / 32];
-    if (lane == 0) part[threadIdx.x >> 5] = sum;
+    __shared__ uint64_t part[S::THREADS / 32];
+    if ((threadIdx.x & 31u) == 0u) part[threadIdx.x >> 5] = sum;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0u) {
         uint64_t t = 0;
 #pragma unroll
-        for (int i = 0; i < kThreads / 32; ++i) t += part[i];
-        atomicAdd(out, static_cast<unsigned long long>(t));
+        for (int i = 0; i < S::THREADS / 32; ++i) t += part[i];
+        if (p.write_src != 0u) *out = t;
+        else atomicAdd(out, static_cast<unsigned long long>(t));
     }
 }
 
@@ -638,8 +547,8 @@ cudaError_t persistent_grid(K kernel, int threads, GridCache& cache, int* grid) 
 // Launches `kernel` on the packed table. A warp takes spans of up to four tiles, so that
 // the lookup of their segment is paid once; fewer where a warp would get less than eight
 // spans, so that all warps end at about the same time.
-template <typename S, typename P, typename K>
-cudaError_t launch(K kernel, GridCache& cache, P& p, int grid_ctas, cudaStream_t stream) {
+template <typename S, typename P, typename K, typename... More>
+cudaError_t launch(K kernel, GridCache& cache, P& p, int grid_ctas, cudaStream_t stream, More... more) {
     int grid = grid_ctas;
     if (grid <= 0) {
         cudaError_t err = persistent_grid(kernel, S::THREADS, cache, &grid);
@@ -650,13 +559,14 @@ cudaError_t launch(K kernel, GridCache& cache, P& p, int grid_ctas, cudaStream_t
     while (p.span > 1 && p.n_tiles < 8 * warps * p.span) p.span /= 2;
     const uint32_t needed = (p.n_tiles + p.span - 1) / p.span;
     if (grid_ctas <= 0 && needed < static_cast<uint32_t>(grid)) grid = static_cast<int>(needed);
-    kernel<<<grid, S::THREADS, 0, stream>>>(p);
+    kernel<<<grid, S::THREADS, 0, stream>>>(p, more...);
     return cudaGetLastError();
 }
 
 template <typename T, bool SMALL, typename P>
 cudaError_t launch_work(const Job& job, P& p) {
-    static GridCache caches[3];
+    static GridCache caches[4];
+    using C = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::Sum>;
     using U = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::Update>;
     using G = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::General>;
     using S = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::Pair>;
@@ -666,6 +576,8 @@ cudaError_t launch_work(const Job& job, P& p) {
             return launch<S>(one_seed_kernel<T, S, kAddToDst, P>, caches[0], p, ctas, job.stream);
         return launch<G>(general_update_kernel<T, G, P>, caches[1], p, ctas, job.stream);
     } else {
+        if (job.work == kChecksum)
+            return launch<C>(checksum_kernel<T, C, P>, caches[3], p, ctas, job.stream, job.sum);
         if (job.work == kPerturb)
             return launch<S>(one_seed_kernel<T, S, kPerturbInPlace, P>, caches[0], p, ctas, job.stream);
         if (p.n_seeds == 1)
@@ -675,12 +587,13 @@ cudaError_t launch_work(const Job& job, P& p) {
 }
 
 // Packs segments, cut at multiples of kPieceElems, into launches whose pieces share the
-// high word of their block indices.
+// high word of their block (checksum: window) indices.
 template <typename T, typename SEG>
 cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size_t n_segs) {
     using P = Launch<SEG, kParamBytes>;
     constexpr uint64_t E = Traits<T>::E, ES = sizeof(T);
-    const uint64_t big_vec = 32ull * (job.n_seeds == 1        ? Traits<T>::Pair::V
+    const uint64_t big_vec = 32ull * (job.work == kChecksum  ? Traits<T>::Sum::V
+                                      : job.n_seeds == 1     ? Traits<T>::Pair::V
                                       : job.work == kGeneral ? Traits<T>::General::V
                                                              : Traits<T>::Update::V);
     uint64_t big_tiles = 0;
@@ -694,13 +607,17 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
     const size_t room = (P::kBytes - p.seg_at) / sizeof(SEG) - 1;  // and the sentinel
     SEG* table = reinterpret_cast<SEG*>(p.data + p.seg_at);
 
+    const uint64_t per_index = job.work == kChecksum ? E : 4;  // elements of a window or block
+    const uint64_t step = job.work == kChecksum ? 1 : E / 4;   // indices of a vector
+    const auto high = [&](uint64_t fo) { return static_cast<uint32_t>((fo / per_index) >> 32); };
     size_t i = 0;
     uint64_t at = 0;  // elements of segs[i] already launched
+    bool cleared = false;
     while (i < n_segs) {
-        const uint32_t hi = static_cast<uint32_t>((segs[i].fo + at) >> 34);
+        const uint32_t hi = high(segs[i].fo + at);
         size_t count = 0;
         uint64_t tiles = 0;
-        while (i < n_segs && count < room && ((segs[i].fo + at) >> 34) == hi && tiles < (1ull << 30)) {
+        while (i < n_segs && count < room && high(segs[i].fo + at) == hi && tiles < (1ull << 30)) {
             const uint64_t fo = segs[i].fo + at;
             const uint64_t n = std::min(segs[i].n - at, kPieceElems - fo % kPieceElems);
             const uint64_t src = segs[i].ptr + at * ES;
@@ -709,7 +626,7 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
             g.head = static_cast<uint32_t>(fo % E);
             g.base = src - g.head * ES;
             g.end = g.head + n;
-            g.blk0 = static_cast<uint32_t>(fo / E * (E / 4));
+            g.blk0 = static_cast<uint32_t>(fo / E * step);
             g.tile0 = static_cast<uint32_t>(tiles);
             // 16-byte vectors line up with element groups whose global index is a
             // multiple of E iff the first window's address is a multiple of 16
@@ -734,15 +651,28 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
         for (int k = 0; k < job.n_seeds; ++k) sp[k] = seed_param(job.seeds[k], hi, job.coef[k]);
         for (int k = 0; k < job.n_groups; ++k) sp[job.group_end[k] - 1].ends_group = 1u;
         cudaError_t err;
+        Job now = job;
+        if (job.work == kChecksum) {
+            p.window_hi = hi;
+            // one CTA (two tiles per warp) instead of several and a cleared sum
+            const bool alone = small && !cleared && i == n_segs && tiles <= 32 && job.grid_ctas <= 0;
+            p.write_src = alone ? 1u : 0u;
+            if (alone) now.grid_ctas = 1;
+            if (!alone && !cleared) {
+                err = cudaMemsetAsync(job.sum, 0, sizeof(*job.sum), job.stream);
+                if (err != cudaSuccess) return err;
+                cleared = true;
+            }
+        }
         const size_t used = p.seg_at + (count + 1) * sizeof(SEG);
         if (!small) {
-            err = launch_work<T, false>(job, p);
+            err = launch_work<T, false>(now, p);
         } else if (used > kSmallParamBytes) {
-            err = launch_work<T, true>(job, p);
+            err = launch_work<T, true>(now, p);
         } else {
             Launch<SEG, kSmallParamBytes> q;
             std::memcpy(&q, &p, offsetof(P, data) + used);
-            err = launch_work<T, true>(job, q);
+            err = launch_work<T, true>(now, q);
         }
         if (err != cudaSuccess) return err;
     }
@@ -758,30 +688,6 @@ cudaError_t enqueue(const Job& job, const Seg* segs, const uint64_t* dst, size_t
     }
     if (job.dtype == kF32) return enqueue_t<float, SegParam>(job, segs, nullptr, n_segs);
     return enqueue_t<__nv_bfloat16, SegParam>(job, segs, nullptr, n_segs);
-}
-
-template <typename T>
-cudaError_t launch_checksum_t(const SumParams& p, unsigned long long* out, int grid_ctas,
-                              cudaStream_t stream) {
-    static GridCache cache;
-    if (p.n_vec == 0) return cudaSuccess;
-    auto kernel = checksum_kernel<T>;
-    int grid = grid_ctas;
-    if (grid <= 0) {
-        cudaError_t err = persistent_grid(kernel, kThreads, cache, &grid);
-        if (err != cudaSuccess) return err;
-        constexpr uint64_t vec_per_cta = 32ull * kSumV * kSumS * (kThreads / 32);
-        const uint64_t needed = (p.n_vec + vec_per_cta - 1) / vec_per_cta;
-        if (needed < static_cast<uint64_t>(grid)) grid = static_cast<int>(needed);
-    }
-    kernel<<<grid, kThreads, 0, stream>>>(p, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_checksum(const SumParams& p, int dtype, unsigned long long* out, int grid_ctas,
-                            cudaStream_t s) {
-    if (dtype == kF32) return launch_checksum_t<float>(p, out, grid_ctas, s);
-    return launch_checksum_t<__nv_bfloat16>(p, out, grid_ctas, s);
 }
 
 static unsigned blocks_for(uint64_t n) { return static_cast<unsigned>((n + 255) / 256); }

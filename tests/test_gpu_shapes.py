@@ -76,6 +76,19 @@ def test_large_shape_equals_small_pieces(jb, dtype, tiles, extra, shift):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("vectors", [1, 31 * 32 + 1, 32 * 32, 32 * 32 + 1, 1600 * 192 - 1, 1600 * 192 + 33])
+def test_checksum_shapes(jb, dtype, vectors):
+    """One CTA that stores its sum, several that add to a cleared one, the large shape."""
+    per = 4 if dtype == "f32" else 8
+    for n, fo in ((vectors * per, 0), (vectors * per - 1, 5), (vectors * per, (1 << 33) - 8)):
+        v = synthetic.normal_values(n, 0.02, 64)
+        v = v if dtype == "f32" else oracle.round_bf16(v.astype(np.float64))
+        out = torch.full((1,), 12345, dtype=torch.int64, device="cuda")
+        jb.jb_checksum(jb.ParamTable([to_device(v)], [fo]), out)
+        assert int(out.item()) & (2**64 - 1) == oracle.checksum([v], [fo])
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("boundary", [1 << 33, 1 << 34, 3 << 33])
 def test_segment_across_a_cut(jb, dtype, boundary):
     """A segment that crosses a multiple of 2^33 elements (2^34: another high word)."""
