@@ -14,7 +14,6 @@
 
 #include "jb.h"
 #include "jb_internal.h"
-#include "jb_q4.h"
 
 #define JB_EXPORT extern "C" __attribute__((visibility("default")))
 
@@ -348,8 +347,7 @@ namespace {
 int perturb_q4_impl(const jb_q4_segment* segs, int n_segs, jb_seed seed, float eps, cudaStream_t stream) {
     if (n_segs < 0 || (n_segs > 0 && segs == nullptr)) return JB_ERR_INVALID_ARG;
     if (!std::isfinite(eps)) return JB_ERR_INVALID_ARG;
-    struct Q { uint64_t codes, scale, fo, n; };
-    std::vector<Q> v;
+    std::vector<jb::Q4Seg> v;
     struct Iv { uint64_t a, b; };
     std::vector<Iv> mem, idx;
     for (int i = 0; i < n_segs; ++i) {
@@ -372,33 +370,7 @@ int perturb_q4_impl(const jb_q4_segment* segs, int n_segs, jb_seed seed, float e
             if ((*list)[i - 1].b > (*list)[i].a) return JB_ERR_INVALID_ARG;
     }
     if (v.empty()) return JB_OK;
-    static thread_local jb::Q4Params params;
-    params.seed = seed_raw(seed);
-    params.eps = eps;
-    for (size_t first = 0; first < v.size(); first += jb::kMaxSegsQ4) {
-        const size_t count = std::min<size_t>(jb::kMaxSegsQ4, v.size() - first);
-        uint64_t unit = 0;
-        params.block_hi = static_cast<uint32_t>(v[first].fo >> 34);
-        params.one_hi = 1;
-        for (size_t i = 0; i < count; ++i) {
-            const Q& q = v[first + i];
-            jb::SegParamQ4& g = params.segs[i];
-            g.codes = q.codes;
-            g.scale = q.scale;
-            g.fo = q.fo;
-            g.n = q.n;
-            g.unit0 = unit;
-            // (a unit past the end of a tensor draws nothing that is kept)
-            if ((q.fo >> 34) != params.block_hi || ((q.fo + q.n - 1) >> 34) != params.block_hi)
-                params.one_hi = 0;
-            unit += jb::kQ4UnitsPerBlock * ((q.n + 63) / 64);  // whole 64-element blocks
-        }
-        params.n_segs = static_cast<uint32_t>(count);
-        params.n_units = unit;
-        const int rc = cuda_status(jb::launch_q4_perturb(params, 0, stream));
-        if (rc != JB_OK) return rc;
-    }
-    return JB_OK;
+    return cuda_status(jb::enqueue_q4(seed_raw(seed), eps, v.data(), v.size(), stream));
 }
 }  // namespace
 

@@ -108,31 +108,35 @@ struct Seg {
 };
 
 // 4-bit weights: codes (two per byte, element 2i in the low nibble) and one fp32
-// scale per 64 elements. A segment owns units [unit0, unit0 + units), kQ4UnitsPerBlock
-// consecutive units per 64-element block (jb_q4.h).
-constexpr int kMaxSegsQ4 = 800;
-
+// scale per 64 elements.
 struct SegParamQ4 {
-    uint64_t codes;  // device address, 8-byte aligned
-    uint64_t scale;  // device address of the fp32 scales
-    uint64_t fo;     // global index of element 0 (a multiple of 4)
+    uint64_t codes;   // device address, 8-byte aligned
+    uint64_t scale;   // device address of the fp32 scales
     uint64_t n;
-    uint64_t unit0;
+    uint32_t blk0;    // Philox block index of element 0 (its global index is a multiple of 4)
+    uint32_t blk_hi;
+    uint32_t tile0;   // first tile (1024 elements each)
+    uint32_t wide;    // the codes are 16-byte aligned
 };
 
-struct Q4Params {
+template <int BYTES>
+struct Q4Launch {
+    static constexpr int kBytes = BYTES;
     SeedRaw seed;
     float eps;
     uint32_t n_segs;
-    uint32_t block_hi;   // high word of the first block index of the launch
-    uint32_t one_hi;     // every block index of the launch has that high word
-    uint64_t n_units;
-    SegParamQ4 segs[kMaxSegsQ4];
+    uint32_t n_tiles;
+    uint32_t span;
+    uint32_t block_hi;  // high word of the block indices where they agree in it
+    alignas(16) unsigned char data[BYTES];
+};
+static_assert(sizeof(Q4Launch<kParamBytes>) <= 32764, "4-bit launch exceeds the parameter space");
+
+struct Q4Seg {
+    uint64_t codes, scale, fo, n;
 };
 
-static_assert(sizeof(Q4Params) <= 32764, "4-bit launch exceeds the parameter space");
-
-cudaError_t launch_q4_perturb(const Q4Params& p, int grid_ctas, cudaStream_t s);
+cudaError_t enqueue_q4(const SeedRaw& seed, float eps, const Q4Seg* segs, size_t n_segs, cudaStream_t stream);
 void q4_levels_host(float out[16]);
 
 enum DType { kF32 = 0, kBF16 = 1 };

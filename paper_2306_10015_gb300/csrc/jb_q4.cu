@@ -25,10 +25,12 @@
 // shared-memory read and one comparison instead of a 4-step binary search.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <atomic>
+#include <cstddef>
+#include <cstring>
 
 #include "jb_internal.h"
-#include "jb_q4.h"
 #include "jb_rng.cuh"
 
 namespace jb {
@@ -46,24 +48,64 @@ __constant__ float c_level[16] = {
     kQ4Level[6], kQ4Level[7], kQ4Level[8],  kQ4Level[9],  kQ4Level[10], kQ4Level[11],
     kQ4Level[12], kQ4Level[13], kQ4Level[14], kQ4Level[15]};
 // midpoints (L_j + L_j+1) / 2 of the fp32 levels, rounded to fp32 (gen_q4_levels.py)
-__constant__ float c_mid[15] = {
+constexpr float kQ4Mid[15] = {
     -0x1.b188d6p-1f, -0x1.374f86p-1f, -0x1.d4b364p-2f, -0x1.59fe86p-2f, -0x1.ddd9e4p-3f,
     -0x1.18df40p-3f, -0x1.72d976p-5f, 0x1.4421acp-5f,  0x1.e9d14cp-4f,  0x1.9e843cp-3f,
     0x1.2969c0p-2f,  0x1.8c97d4p-2f,  0x1.ff3a68p-2f,  0x1.47c276p-1f,  0x1.b8654cp-1f};
 
-// Buckets: bucket[j] for j < 32 = (the midpoint in [(j - 16)/16, (j - 15)/16) or
-// +inf, the number of midpoints below (j - 16)/16 as integer bits); bucket[32 .. 63]
-// = (+inf, 15), for x = 1. For x in [-1, 1], y = x 2^-16 + 1 + 2^-16 rounded toward
-// minus infinity lies in [1, 1 + 2^-15], and its fraction bits 3 .. 8 are
-// floor(16 (x + 1)): the exact value is 1 + 128 (x + 1) 2^-23, every multiple of
-// 2^-20 there is representable, so rounding down never crosses one. The mask gives
-// the byte offset of the 8-byte entry directly; a NaN x gets an unspecified code.
-constexpr float kQ4IdxBias = 0x1.0001p+0f;  // 1 + 2^-16
+// Buckets: entry j < 32 = (the midpoint in [(j - 16)/16, (j - 15)/16) or +inf, the number
+// of midpoints below (j - 16)/16 in each of the eight nibbles); entries 32 .. 63 = (+inf,
+// 15), for x = 1. For x in [-1, 1], y = x 2^-12 + 1 + 2^-12 rounded toward minus infinity
+// lies in [1, 1 + 2^-11], and its fraction bits 7 .. 12 are floor(16 (x + 1)): the exact
+// value is 1 + 2^11 (x + 1) 2^-23, every multiple of 2^-16 there is representable, so
+// rounding down never crosses one. The mask gives the byte offset of a row of 16 equal
+// 8-byte entries, one for each lane of a half warp: a 64-bit read serves half a warp at a
+// time, so no two lanes meet in a bank. A NaN x gets an unspecified code.
+constexpr float kQ4IdxScale = 0x1p-12f, kQ4IdxBias = 0x1.001p+0f;  // 1 + 2^-12
+constexpr int kBucketRow = 16;
+constexpr int kQ4Epl = 32;  // elements per lane and tile
 
-__device__ __forceinline__ uint32_t q4_code(float x, float y, const float2* bucket) {
-    const uint32_t off = __float_as_uint(y) & 0x1F8u;
+struct Bucket {
+    float mid;
+    uint32_t below;
+};
+struct Buckets {
+    Bucket b[64];
+};
+constexpr Buckets make_buckets() {
+    Buckets t{};
+    for (int j = 0; j < 64; ++j) {
+        const float lo = static_cast<float>(j - 16) * 0.0625f;
+        uint32_t below = 0;
+        t.b[j].mid = __builtin_inff();
+        for (int k = 0; k < 15; ++k) {
+            if (kQ4Mid[k] < lo) ++below;
+            if (kQ4Mid[k] >= lo && kQ4Mid[k] < lo + 0.0625f) t.b[j].mid = kQ4Mid[k];
+        }
+        t.b[j].below = below * 0x11111111u;
+    }
+    return t;
+}
+__constant__ Buckets c_bucket = make_buckets();
+
+// ow with nibble K replaced by the code of x. The count of midpoints is there in every
+// nibble and x above the bucket's own midpoint adds one in nibble K (a count is at most 14
+// where a midpoint can lie above), so a code costs a comparison, a predicated addition and
+// one bitwise select, and no shift; shifting each code into place cost 14 instructions of
+// the integer-multiply pipe per four elements, the pipe that bounds this kernel.
+template <int K>
+__device__ __forceinline__ uint32_t put_code(uint32_t ow, float x, float y, const float2* bucket,
+                                             uint32_t lane_off) {
+    uint32_t off;
+    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(off) : "r"(__float_as_uint(y)), "r"(0x1F80u), "r"(lane_off));
     const float2 e = *reinterpret_cast<const float2*>(reinterpret_cast<const char*>(bucket) + off);
-    return __float_as_uint(e.y) + (x > e.x ? 1u : 0u);
+    uint32_t v = __float_as_uint(e.y);
+    asm("{\n\t.reg .pred p;\n\tsetp.gt.f32 p, %1, %2;\n\t@p add.u32 %0, %0, %3;\n\t}"
+        : "+r"(v) : "f"(x), "f"(e.x), "n"(1u << (4 * K)));
+    if constexpr (K == 0) return v;
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, 0xE4;" : "=r"(r) : "r"(v), "r"(ow), "r"(0xFu << (4 * K)));
+    return r;
 }
 
 // max(a, b, c) in one instruction
@@ -91,183 +133,198 @@ __device__ __forceinline__ void dequant_block(const float2* pair, const uint32_t
     lo = pair_at<B % 2, true>(pair, cw[B / 2]);
 }
 
-constexpr int kThreadsQ4 = 512;
+constexpr int kThreadsQ4 = 768;
 
-// 64 registers: two CTAs per SM, measured 2.7% faster than the compiler's 70 registers
-// and one CTA. ONE_HI: the pair's constants hold for every block of the launch;
-// otherwise they are formed for the high word of each lane's own block index.
-template <bool ONE_HI>
-__global__ void __maxnreg__(64) q4_perturb_kernel(const __grid_constant__ Q4Params p) {
+template <typename P>
+__device__ __forceinline__ const SegParamQ4& q4_seg(const P& p, uint32_t s) {
+    return reinterpret_cast<const SegParamQ4*>(p.data)[s];
+}
+
+// A warp tile is 1024 consecutive elements of one tensor, 32 per lane; tiles and spans as
+// in the update's kernels. Bound, like those, by operand reads and the instruction mix
+// (139 instructions and 229 cycles per scheduler and four elements of a warp; FMA pipe 73%
+// busy, shared-memory reads 39%). Six warps per scheduler at 80 registers: 2^28 elements
+// in 357 us (640 threads 363, 1024 threads 360, 512 threads 371); 397 before, with lanes
+// numbered across tensors, codes shifted into place and bank conflicts on the buckets.
+// ONE_HI: the pair's constants hold for every block of the launch; otherwise they are
+// formed for the high word of each block's own index.
+template <bool ONE_HI, typename P>
+__global__ void __launch_bounds__(kThreadsQ4) q4_perturb_kernel(const __grid_constant__ P p) {
     constexpr int E = kQ4Epl, NB = E / 4, NW = E / 8;
-    static_assert(kQ4UnitsPerBlock == 2 && NB == 8, "two 32-element lanes per block");
+    static_assert(NB == 8 && 64 == 2 * E, "two 32-element lanes per scale block");
     __shared__ float2 pair[kPairEntries];
-    __shared__ float2 bucket[64];
+    __shared__ float2 bucket[64 * kBucketRow];
     for (int i = threadIdx.x; i < 256; i += kThreadsQ4)
         pair[(i & 15) + 256 * (i >> 4)] = make_float2(c_level[i & 15], c_level[i >> 4]);
-    if (threadIdx.x >= 32 && threadIdx.x < 64)
-        bucket[threadIdx.x] = make_float2(__int_as_float(0x7F800000), __uint_as_float(15u));
-    if (threadIdx.x < 32) {
-        const float lo = static_cast<float>(static_cast<int>(threadIdx.x) - 16) * 0.0625f;
-        const float hi = lo + 0.0625f;
-        uint32_t below = 0;
-        float m = __int_as_float(0x7F800000);  // +inf: no midpoint in the bucket
-#pragma unroll
-        for (int k = 0; k < 15; ++k) {
-            const float md = c_mid[k];
-            below += md < lo ? 1u : 0u;
-            if (md >= lo && md < hi) m = md;
-        }
-        bucket[threadIdx.x] = make_float2(m, __uint_as_float(below));
+    for (int i = threadIdx.x; i < 64 * kBucketRow; i += kThreadsQ4) {
+        const Bucket b = c_bucket.b[i / kBucketRow];
+        bucket[i] = make_float2(b.mid, __uint_as_float(b.below));
     }
     __syncthreads();  // every thread reaches this before any work
 
     const uint32_t lane = threadIdx.x & 31u;
-    const uint64_t warp = (static_cast<uint64_t>(blockIdx.x) * kThreadsQ4 + threadIdx.x) >> 5;
-    const uint64_t n_warps = (static_cast<uint64_t>(gridDim.x) * kThreadsQ4) >> 5;
+    const uint32_t lane_off = 8u * (lane % kBucketRow);
     SeedParam sc = seed_param(p.seed, p.block_hi, p.eps);
     const float2 eps2 = splat(p.eps);
-    uint32_t s = 0;
+    const uint64_t span = p.span;
+    const uint64_t stride = span * (static_cast<uint64_t>(gridDim.x) * (kThreadsQ4 / 32));
+    uint32_t s = 0;  // tensor cursor; only moves forward
     // all 32 lanes run every iteration (the block maximum is a warp shuffle)
-    for (uint64_t wt = warp; wt * 32u < p.n_units; wt += n_warps) {
-        const uint64_t unit = wt * 32u + lane;
-        const bool valid = unit < p.n_units;
-        if (valid)
-            while (s + 1 < p.n_segs && p.segs[s + 1].unit0 <= unit) ++s;
-        const SegParamQ4& g = p.segs[s];
-        const uint64_t u = unit - g.unit0;
-        const int64_t i0 = static_cast<int64_t>(E * u);
-        const int64_t n = static_cast<int64_t>(g.n);
-        const bool any = valid && i0 < n;
-        const bool full = valid && i0 + E <= n;
-        uint8_t* codes = reinterpret_cast<uint8_t*>(g.codes);
-        float* scale = reinterpret_cast<float*>(g.scale);
+    for (uint64_t t0 = span * (static_cast<uint64_t>(threadIdx.x >> 5) * gridDim.x + blockIdx.x);
+         t0 < p.n_tiles; t0 += stride) {
+        const uint32_t t_end = static_cast<uint32_t>(t0 + span < p.n_tiles ? t0 + span : p.n_tiles);
+        for (uint32_t t = static_cast<uint32_t>(t0); t < t_end; ++t) {
+            if (t >= q4_seg(p, s + 1).tile0) {
+                uint32_t lo = s + 1, hi = p.n_segs;
+                while (hi - lo > 1) {
+                    const uint32_t m = (lo + hi) / 2;
+                    if (q4_seg(p, m).tile0 <= t) lo = m;
+                    else hi = m;
+                }
+                s = lo;
+            }
+            const SegParamQ4& g = q4_seg(p, s);
+            const uint64_t first = static_cast<uint64_t>(t - g.tile0) * (32u * E);
+            const uint64_t i0 = first + E * lane;
+            const bool fast = first + 32u * E <= g.n;  // the same for every lane
+            const bool any = fast || i0 < g.n;
+            const bool full = fast || i0 + E <= g.n;
+            uint8_t* codes = reinterpret_cast<uint8_t*>(g.codes) + i0 / 2;
+            float* scale = reinterpret_cast<float*>(g.scale) + i0 / 64;
 
-        uint32_t cw[NW];  // 32 codes, 8 per word
+            uint32_t cw[NW];  // 32 codes, 8 per word
 #pragma unroll
-        for (int j = 0; j < NW; ++j) cw[j] = 0u;
-        if (full) {
+            for (int j = 0; j < NW; ++j) cw[j] = 0u;
+            if (full) {
+                if (g.wide) {
+                    const uint4 v = __ldcs(reinterpret_cast<const uint4*>(codes));
+                    cw[0] = v.x; cw[1] = v.y; cw[2] = v.z; cw[3] = v.w;
+                } else {
 #pragma unroll
-            for (int j = 0; j < NW; j += 2) {  // codes are 8-byte aligned
-                const uint2 v = *reinterpret_cast<const uint2*>(codes + i0 / 2 + 4 * j);
-                cw[j] = v.x;
-                cw[j + 1] = v.y;
+                    for (int j = 0; j < NW; j += 2) {  // codes are 8-byte aligned
+                        const uint2 v = *reinterpret_cast<const uint2*>(codes + 4 * j);
+                        cw[j] = v.x;
+                        cw[j + 1] = v.y;
+                    }
+                }
+            } else if (any) {
+#pragma unroll
+                for (int b = 0; b < E / 2; ++b)
+                    if (i0 + 2 * b < g.n) cw[b / 4] |= static_cast<uint32_t>(codes[b]) << (8 * (b % 4));
             }
-        } else if (any) {
-#pragma unroll
-            for (int b = 0; b < E / 2; ++b)
-                if (i0 + 2 * b < n) cw[b / 4] |= static_cast<uint32_t>(codes[i0 / 2 + b]) << (8 * (b % 4));
-        }
-        const float2 s2 = splat(any ? scale[u >> 1] : 0.0f);
+            const float2 s2 = splat(any ? *scale : 0.0f);
 
-        // dequantize and perturb: w = fma(cos or sin, eps r, level * scale), the
-        // Philox words of block b + 1 computed while block b is transformed;
-        // wv[2b] = elements (4b, 4b + 2), wv[2b + 1] = (4b + 1, 4b + 3)
-        float2 wv[E / 2];
-        const uint64_t blk0 = (g.fo + static_cast<uint64_t>(i0)) >> 2;  // fo % 4 == 0
-        const uint32_t blk = static_cast<uint32_t>(blk0);
-        uint4 wcur;
-        if constexpr (!ONE_HI) sc = seed_param(p.seed, static_cast<uint32_t>(blk0 >> 32), p.eps);
-        wcur = philox_block(sc, blk);
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            uint4 wnext;
-            if (b + 1 < NB) {
-                if constexpr (!ONE_HI)
-                    sc = seed_param(p.seed, static_cast<uint32_t>((blk0 + b + 1) >> 32), p.eps);
-                wnext = philox_block(sc, blk + b + 1);
-            }
-            const Polar2 o = polar2(wcur);
-            if (b + 1 < NB) wcur = wnext;
-            const float2 rc = mul2(eps2, o.rr);
-            float2 le, lo;
-            switch (b) {
-                case 0: dequant_block<0>(pair, cw, le, lo); break;
-                case 1: dequant_block<1>(pair, cw, le, lo); break;
-                case 2: dequant_block<2>(pair, cw, le, lo); break;
-                case 3: dequant_block<3>(pair, cw, le, lo); break;
-                case 4: dequant_block<4>(pair, cw, le, lo); break;
-                case 5: dequant_block<5>(pair, cw, le, lo); break;
-                case 6: dequant_block<6>(pair, cw, le, lo); break;
-                default: dequant_block<7>(pair, cw, le, lo); break;
-            }
-            wv[2 * b] = fma2(o.cm, rc, mul2(le, s2));
-            wv[2 * b + 1] = fma2(o.sm, rc, mul2(lo, s2));
-        }
-        // elements past the end of the segment do not count towards the maximum
-        if (!full) {
+            // dequantize and perturb: w = fma(cos or sin, eps r, level * scale), the
+            // Philox words of block b + 1 computed while block b is transformed;
+            // wv[2b] = elements (4b, 4b + 2), wv[2b + 1] = (4b + 1, 4b + 3)
+            float2 wv[E / 2];
+            const uint32_t blk = g.blk0 + static_cast<uint32_t>(i0 >> 2);
+            const auto words = [&](int b) {
+                if constexpr (!ONE_HI) {
+                    const uint64_t at = ((static_cast<uint64_t>(g.blk_hi) << 32) | g.blk0) + (i0 >> 2) + b;
+                    sc = seed_param(p.seed, static_cast<uint32_t>(at >> 32), p.eps);
+                }
+                return philox_block(sc, blk + b);
+            };
+            uint4 wcur = words(0);
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
-                if (i0 + 4 * b + 0 >= n) wv[2 * b].x = 0.0f;
-                if (i0 + 4 * b + 2 >= n) wv[2 * b].y = 0.0f;
-                if (i0 + 4 * b + 1 >= n) wv[2 * b + 1].x = 0.0f;
-                if (i0 + 4 * b + 3 >= n) wv[2 * b + 1].y = 0.0f;
+                uint4 wnext;
+                if (b + 1 < NB) wnext = words(b + 1);
+                const Polar2 o = polar2(wcur);
+                if (b + 1 < NB) wcur = wnext;
+                const float2 rc = mul2(eps2, o.rr);
+                float2 le, lo;
+                if (b % 2 == 0) dequant_block<0>(pair, cw + b / 2, le, lo);
+                else dequant_block<1>(pair, cw + b / 2, le, lo);
+                wv[2 * b] = fma2(o.cm, rc, mul2(le, s2));
+                wv[2 * b + 1] = fma2(o.sm, rc, mul2(lo, s2));
             }
-        }
-        float m = 0.0f;
+            // elements past the end of the tensor do not count towards the maximum
+            if (!full) {
 #pragma unroll
-        for (int i = 0; i < E / 2; ++i) m = fmax3(m, fabsf(wv[i].x), fabsf(wv[i].y));
-        // block maximum over the two lanes of the block (lanes 2j, 2j + 1)
-        m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
-        // 1/m rounded down: every |w / m| then rounds to at most 1, so x needs no clamp
-        const float2 inv2 = splat(m > 0.0f ? __frcp_rd(m) : 0.0f);
+                for (int b = 0; b < NB; ++b) {
+                    if (i0 + 4 * b + 0 >= g.n) wv[2 * b].x = 0.0f;
+                    if (i0 + 4 * b + 2 >= g.n) wv[2 * b].y = 0.0f;
+                    if (i0 + 4 * b + 1 >= g.n) wv[2 * b + 1].x = 0.0f;
+                    if (i0 + 4 * b + 3 >= g.n) wv[2 * b + 1].y = 0.0f;
+                }
+            }
+            float m = 0.0f;
+#pragma unroll
+            for (int i = 0; i < E / 2; ++i) m = fmax3(m, fabsf(wv[i].x), fabsf(wv[i].y));
+            // block maximum over the two lanes of the block (lanes 2j, 2j + 1)
+            m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
+            // 1/m rounded down: every |w / m| then rounds to at most 1, so x needs no clamp
+            const float2 inv2 = splat(m > 0.0f ? __frcp_rd(m) : 0.0f);
 
-        // quantize again: x = w / m, its bucket from y = RD(x 2^-16 + 1 + 2^-16)
-        uint32_t ow[NW];
+            // quantize again: x = w / m, its bucket from y = RD(x 2^-12 + 1 + 2^-12)
+            uint32_t ow[NW];
 #pragma unroll
-        for (int j = 0; j < NW; ++j) ow[j] = 0u;
+            for (int j = 0; j < NW; ++j) {
+                float2 x[4], y[4];  // elements (0, 2), (1, 3), (4, 6), (5, 7) of the word
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float2 x = mul2(wv[2 * b + h], inv2);
-                const float2 y = __ffma2_rd(x, splat(0x1p-16f), splat(kQ4IdxBias));
-                const int ka = 4 * b + h, kb = 4 * b + h + 2;
-                ow[ka / 8] += q4_code(x.x, y.x, bucket) << (4 * (ka % 8));
-                ow[kb / 8] += q4_code(x.y, y.y, bucket) << (4 * (kb % 8));
+                for (int h = 0; h < 4; ++h) {
+                    x[h] = mul2(wv[4 * j + h], inv2);
+                    y[h] = __ffma2_rd(x[h], splat(kQ4IdxScale), splat(kQ4IdxBias));
+                }
+                uint32_t o = put_code<0>(0u, x[0].x, y[0].x, bucket, lane_off);
+                o = put_code<1>(o, x[1].x, y[1].x, bucket, lane_off);
+                o = put_code<2>(o, x[0].y, y[0].y, bucket, lane_off);
+                o = put_code<3>(o, x[1].y, y[1].y, bucket, lane_off);
+                o = put_code<4>(o, x[2].x, y[2].x, bucket, lane_off);
+                o = put_code<5>(o, x[3].x, y[3].x, bucket, lane_off);
+                o = put_code<6>(o, x[2].y, y[2].y, bucket, lane_off);
+                ow[j] = put_code<7>(o, x[3].y, y[3].y, bucket, lane_off);
             }
-        }
-        if (full) {
+            if (full) {
+                if (g.wide) {
+                    __stcs(reinterpret_cast<uint4*>(codes), make_uint4(ow[0], ow[1], ow[2], ow[3]));
+                } else {
 #pragma unroll
-            for (int j = 0; j < NW; j += 2)
-                *reinterpret_cast<uint2*>(codes + i0 / 2 + 4 * j) = make_uint2(ow[j], ow[j + 1]);
-        } else if (any) {
+                    for (int j = 0; j < NW; j += 2)
+                        *reinterpret_cast<uint2*>(codes + 4 * j) = make_uint2(ow[j], ow[j + 1]);
+                }
+            } else if (any) {
 #pragma unroll
-            for (int b = 0; b < E / 2; ++b) {
-                if (i0 + 2 * b >= n) continue;
-                const uint8_t byte = static_cast<uint8_t>(ow[b / 4] >> (8 * (b % 4)));
-                // an odd tail leaves the unused high nibble of the last byte as it was
-                codes[i0 / 2 + b] = (i0 + 2 * b + 1 < n) ? byte
-                                                         : static_cast<uint8_t>((codes[i0 / 2 + b] & 0xF0u) | (byte & 0x0Fu));
+                for (int b = 0; b < E / 2; ++b) {
+                    if (i0 + 2 * b >= g.n) continue;
+                    const uint8_t byte = static_cast<uint8_t>(ow[b / 4] >> (8 * (b % 4)));
+                    // an odd tail leaves the unused high nibble of the last byte as it was
+                    codes[b] = (i0 + 2 * b + 1 < g.n) ? byte
+                                                      : static_cast<uint8_t>((codes[b] & 0xF0u) | (byte & 0x0Fu));
+                }
             }
+            if (any && (lane & 1u) == 0u) *scale = m;
         }
-        if (any && (u & 1u) == 0u) scale[u >> 1] = m;
     }
 }
 
-std::atomic<int> g_q4_grid[2][64];
+std::atomic<int> g_q4_grid[64][4];
 
-template <bool ONE_HI>
-cudaError_t launch_q4_t(const Q4Params& p, int grid_ctas, cudaStream_t stream) {
-    int grid = grid_ctas;
+template <bool ONE_HI, typename P>
+cudaError_t launch_q4(P& p, int slot, cudaStream_t stream) {
+    auto kernel = q4_perturb_kernel<ONE_HI, P>;
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return err;
+    int grid = dev < 64 ? g_q4_grid[dev][slot].load(std::memory_order_relaxed) : 0;
     if (grid <= 0) {
-        int dev = 0;
-        cudaError_t err = cudaGetDevice(&dev);
+        int sms = 0, per_sm = 0;
+        err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (err != cudaSuccess) return err;
-        grid = dev < 64 ? g_q4_grid[ONE_HI][dev].load(std::memory_order_relaxed) : 0;
-        if (grid <= 0) {
-            int sms = 0, per_sm = 0;
-            err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (err != cudaSuccess) return err;
-            err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, q4_perturb_kernel<ONE_HI>,
-                                                                kThreadsQ4, 0);
-            if (err != cudaSuccess) return err;
-            grid = sms * (per_sm > 0 ? per_sm : 1);
-            if (dev < 64) g_q4_grid[ONE_HI][dev].store(grid, std::memory_order_relaxed);
-        }
-        const uint64_t needed = (p.n_units + kThreadsQ4 - 1) / kThreadsQ4;
-        if (needed < static_cast<uint64_t>(grid)) grid = static_cast<int>(needed);
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreadsQ4, 0);
+        if (err != cudaSuccess) return err;
+        grid = sms * (per_sm > 0 ? per_sm : 1);
+        if (dev < 64) g_q4_grid[dev][slot].store(grid, std::memory_order_relaxed);
     }
-    q4_perturb_kernel<ONE_HI><<<grid, kThreadsQ4, 0, stream>>>(p);
+    // spans as in the update's launches
+    const uint64_t warps = static_cast<uint64_t>(grid) * (kThreadsQ4 / 32);
+    p.span = 4;
+    while (p.span > 1 && p.n_tiles < 8 * warps * p.span) p.span /= 2;
+    const uint32_t needed = (p.n_tiles + p.span - 1) / p.span;
+    if (needed < static_cast<uint32_t>(grid)) grid = static_cast<int>(needed);
+    kernel<<<grid, kThreadsQ4, 0, stream>>>(p);
     return cudaGetLastError();
 }
 
@@ -277,9 +334,55 @@ void q4_levels_host(float out[16]) {
     for (int i = 0; i < 16; ++i) out[i] = kQ4Level[i];
 }
 
-cudaError_t launch_q4_perturb(const Q4Params& p, int grid_ctas, cudaStream_t stream) {
-    if (p.n_units == 0) return cudaSuccess;
-    return p.one_hi ? launch_q4_t<true>(p, grid_ctas, stream) : launch_q4_t<false>(p, grid_ctas, stream);
+cudaError_t enqueue_q4(const SeedRaw& seed, float eps, const Q4Seg* segs, size_t n_segs, cudaStream_t stream) {
+    using P = Q4Launch<kParamBytes>;
+    static thread_local P p;  // ~32 KB: keep it off the stack
+    p.seed = seed;
+    p.eps = eps;
+    constexpr size_t room = P::kBytes / sizeof(SegParamQ4) - 1;  // and the sentinel
+    SegParamQ4* table = reinterpret_cast<SegParamQ4*>(p.data);
+    size_t i = 0;
+    uint64_t at = 0;  // elements of segs[i] already launched
+    while (i < n_segs) {
+        size_t count = 0;
+        uint64_t tiles = 0;
+        bool one_hi = true;
+        p.block_hi = static_cast<uint32_t>((segs[i].fo + at) >> 34);
+        while (i < n_segs && count < room && tiles < (1ull << 30)) {
+            const uint64_t n = std::min<uint64_t>(segs[i].n - at, 1ull << 40);  // keeps a tile number in 32 bits
+            const uint64_t fo = segs[i].fo + at;
+            SegParamQ4& g = table[count++];
+            g.codes = segs[i].codes + at / 2;
+            g.scale = segs[i].scale + at / 64 * 4;
+            g.n = n;
+            g.blk0 = static_cast<uint32_t>(fo >> 2);
+            g.blk_hi = static_cast<uint32_t>(fo >> 34);
+            g.tile0 = static_cast<uint32_t>(tiles);
+            g.wide = (g.codes & 15ull) == 0 ? 1u : 0u;
+            // (a lane past the end of a tensor draws nothing that is kept)
+            if ((fo >> 34) != p.block_hi || ((fo + n - 1) >> 34) != p.block_hi) one_hi = false;
+            tiles += (n + 32 * kQ4Epl - 1) / (32 * kQ4Epl);
+            at += n;
+            if (at == segs[i].n) {
+                ++i;
+                at = 0;
+            }
+        }
+        table[count].tile0 = static_cast<uint32_t>(tiles);
+        p.n_segs = static_cast<uint32_t>(count);
+        p.n_tiles = static_cast<uint32_t>(tiles);
+        cudaError_t err;
+        const size_t used = (count + 1) * sizeof(SegParamQ4);
+        if (used <= kSmallParamBytes) {
+            Q4Launch<kSmallParamBytes> q;
+            std::memcpy(&q, &p, offsetof(P, data) + used);
+            err = one_hi ? launch_q4<true>(q, 0, stream) : launch_q4<false>(q, 1, stream);
+        } else {
+            err = one_hi ? launch_q4<true>(p, 2, stream) : launch_q4<false>(p, 3, stream);
+        }
+        if (err != cudaSuccess) return err;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace jb
