@@ -71,7 +71,8 @@ template <typename T>
 struct Traits;
 template <>
 struct Traits<float> {
-    static constexpr int E = 4;  // elements per 16-byte vector
+    static constexpr int E = 4;                     // elements per 16-byte vector
+    static constexpr uint64_t SPLIT_TILES = 608;    // most 128-element tiles of the split update
     using Update = Shape<5, 512, 2>;
     using General = Shape<4, 512, 2>;
     using Pair = Shape<4, 1024, 1>;
@@ -81,6 +82,7 @@ struct Traits<float> {
 template <>
 struct Traits<__nv_bfloat16> {
     static constexpr int E = 8;
+    static constexpr uint64_t SPLIT_TILES = 1216;
     using Update = Shape<3, 512, 2>;
     using General = Shape<2, 512, 2>;
     using Pair = Shape<4, 1024, 1>;
@@ -403,6 +405,149 @@ __global__ void __launch_bounds__(S::THREADS) general_update_kernel(const __grid
     });
 }
 
+// The update of a table so small that its elements cannot fill the GPU: the pairs are
+// shared out too. A group of G warps takes one tile of 128 elements (a Philox block per
+// lane); warp w forms the scaled radii and the signed cosines and sines of pairs w, w + G,
+// ... of a chunk of 2 G pairs in shared memory, and the group's first warp adds them up in
+// pair order, chunk c while the group forms chunk c + 1. The additions are those of
+// update_tile, so the results are the same bit for bit. One warp alone needs about 350
+// cycles per pair for a tile (the latency of the generator and the transform; 580 where a
+// thread has the two blocks of a bf16 vector); shared out, an SM needs about 40. K = 400
+// update, us, before and with the split: fp32 1K to 19K elements 68 and 27, 65K 84 and 53,
+// 78K 84 and 93; bf16 1K 115 and 31, 65K 115 and 53, 160K 148 and 117, 262K 148 and 175.
+// So it ends at one tile per scheduler (608) in fp32 and at two in bf16. It is not slower
+// for two pairs either (4.9 -> 3.3 us for 1K bf16 elements).
+constexpr int kSplitThreads = 512;
+constexpr int kSplitWarps = kSplitThreads / 32;
+constexpr int kSplitPairs = 2;
+
+struct Drawn {
+    float2 rc[32], cm[32], sm[32];  // of one pair, by lane
+};
+
+template <int ES>
+__device__ __forceinline__ void load_block(uint64_t a, int first, int last, bool full, float (&x)[4]) {
+    if constexpr (ES == 4) {
+        if (full) {
+            const float4 v = __ldcs(reinterpret_cast<const float4*>(a));
+            x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+            return;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = i >= first && i < last ? reinterpret_cast<const float*>(a)[i] : 0.0f;
+    } else {
+        uint32_t b[4];
+        if (full) {
+            const uint2 v = __ldcs(reinterpret_cast<const uint2*>(a));
+            b[0] = v.x << 16; b[1] = v.x & 0xFFFF0000u; b[2] = v.y << 16; b[3] = v.y & 0xFFFF0000u;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                b[i] = i >= first && i < last ? static_cast<uint32_t>(reinterpret_cast<const uint16_t*>(a)[i]) << 16 : 0u;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = __uint_as_float(b[i]);
+    }
+}
+
+template <int ES>
+__device__ __forceinline__ void store_block(uint64_t a, int first, int last, bool full, const float (&x)[4]) {
+    if constexpr (ES == 4) {
+        if (full) {
+            __stcs(reinterpret_cast<float4*>(a), make_float4(x[0], x[1], x[2], x[3]));
+            return;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i >= first && i < last) reinterpret_cast<float*>(a)[i] = x[i];
+    } else {
+        const uint32_t lo = pack_bf16(x[0], x[1]), hi = pack_bf16(x[2], x[3]);
+        if (full) {
+            __stcs(reinterpret_cast<uint2*>(a), make_uint2(lo, hi));
+            return;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i >= first && i < last)
+                reinterpret_cast<uint16_t*>(a)[i] = static_cast<uint16_t>((i < 2 ? lo : hi) >> (16 * (i % 2)));
+    }
+}
+
+template <typename T, bool TO_DST, typename P>
+__global__ void __launch_bounds__(kSplitThreads) split_update_kernel(const __grid_constant__ P p) {
+    constexpr int ES = sizeof(T);
+    __shared__ Drawn drawn[4 * kSplitWarps];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t G = p.span;  // warps of a group: 4, 8 or 16
+    const uint32_t group = warp / G, w = warp % G, groups = kSplitWarps / G;
+    Drawn* const buf = drawn + group * (4 * G);  // two chunks of 2 G pairs
+    const uint32_t K = p.n_seeds, chunks = (K + 2 * G - 1) / (2 * G);
+    uint32_t s = 0;
+    // a group's warps see the same tiles: each reaches every barrier of its group
+    for (uint64_t t = static_cast<uint64_t>(group) * gridDim.x + blockIdx.x; t < p.n_tiles;
+         t += static_cast<uint64_t>(groups) * gridDim.x) {
+        s = find_seg(p, s, static_cast<uint32_t>(t));
+        const auto& g = seg_at(p, s);
+        const uint32_t v = (static_cast<uint32_t>(t) - g.tile0) * 32u + lane;
+        const uint32_t blk = g.blk0 + v;
+        const BlockCtr bc = block_ctr(blk);
+        const auto form = [&](uint32_t c) {
+            Drawn* const to = buf + (c & 1u) * (2 * G);
+#pragma unroll
+            for (uint32_t r = 0; r < 2; ++r) {
+                const uint32_t k = c * (2 * G) + r * G + w;
+                if (k >= K) break;
+                const SeedParam& sd = seed_at(p, k);
+                const Polar2 o = polar2(philox_block(sd, bc));
+                Drawn& d = to[r * G + w];
+                d.rc[lane] = mul2(splat(sd.coef), o.rr);
+                d.cm[lane] = o.cm;
+                d.sm[lane] = o.sm;
+            }
+        };
+        // the first warp holds theta and the sum: (elements 0, 2) and (1, 3) of the block
+        const uint64_t e0 = 4ull * v;
+        const int first = v == 0u ? static_cast<int>(g.head) : 0;
+        const int last = e0 >= g.end ? 0 : (g.end - e0 < 4 ? static_cast<int>(g.end - e0) : 4);
+        const bool full = v >= (g.head != 0u ? 1u : 0u) && v < g.full;
+        const uint64_t src = g.base + 4ull * ES * v;
+        float x[4];
+        float2 even = make_float2(0.0f, 0.0f), odd = even;
+        if (w == 0u) load_block<ES>(src, first, last, full, x);
+        form(0);
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(32 * G) : "memory");
+        for (uint32_t c = 0; c < chunks; ++c) {
+            if (w == 0u) {
+                const Drawn* const from = buf + (c & 1u) * (2 * G);
+                const uint32_t n = K - c * (2 * G) < 2 * G ? K - c * (2 * G) : 2 * G;
+#pragma unroll 8
+                for (uint32_t i = 0; i < n; ++i) {
+                    const float2 rc = from[i].rc[lane];
+                    even = fma2(from[i].cm[lane], rc, even);
+                    odd = fma2(from[i].sm[lane], rc, odd);
+                    if (seed_at(p, c * (2 * G) + i).ends_group != 0u) {
+                        x[0] = __fadd_rn(x[0], even.x);
+                        x[2] = __fadd_rn(x[2], even.y);
+                        x[1] = __fadd_rn(x[1], odd.x);
+                        x[3] = __fadd_rn(x[3], odd.y);
+                        if constexpr (ES == 2) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) x[j] = __bfloat162float(__float2bfloat16_rn(x[j]));
+                        }
+                        even = odd = make_float2(0.0f, 0.0f);
+                    }
+                }
+            }
+            if (c + 1 < chunks) form(c + 1);
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(32 * G) : "memory");
+        }
+        if (w == 0u) {
+            store_block<ES>(dst_of(g) + 4ull * ES * v, first, last, full, x);
+            if (TO_DST && p.write_src != 0u) store_block<ES>(src, first, last, full, x);
+        }
+    }
+}
+
 // Model checksum (ChecksumMatch, Algorithm 1): the sum mod 2^64, over 16-byte
 // windows of the global element space, of four Philox rounds of the window's
 // storage words (elements outside the segment read as 0) keyed by the window
@@ -563,6 +708,24 @@ cudaError_t launch(K kernel, GridCache& cache, P& p, int grid_ctas, cudaStream_t
     return cudaGetLastError();
 }
 
+// Tiles of the split update on `sms` SMs go to groups of 16, 8 or 4 warps, so that the
+// CTAs, one per SM, have about one group per tile.
+template <typename T, typename P>
+cudaError_t launch_split(const Job& job, P& p) {
+    static GridCache cache;
+    auto kernel = split_update_kernel<T, std::is_same<typename P::Seg, SegParamOut>::value, P>;
+    int sms = 0;
+    cudaError_t err = persistent_grid(kernel, kSplitThreads, cache, &sms);
+    if (err != cudaSuccess) return err;
+    const uint32_t ctas = static_cast<uint32_t>(job.grid_ctas > 0 ? job.grid_ctas : sms);
+    p.span = p.n_tiles <= ctas ? 16u : p.n_tiles <= 2u * ctas ? 8u : 4u;
+    const uint32_t groups = kSplitWarps / p.span;
+    int grid = static_cast<int>(std::min(ctas, (p.n_tiles + groups - 1) / groups));
+    if (job.grid_ctas > 0) grid = job.grid_ctas;
+    kernel<<<grid, kSplitThreads, 0, job.stream>>>(p);
+    return cudaGetLastError();
+}
+
 template <typename T, bool SMALL, typename P>
 cudaError_t launch_work(const Job& job, P& p) {
     static GridCache caches[4];
@@ -599,7 +762,14 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
     uint64_t big_tiles = 0;
     for (size_t k = 0; k < n_segs; ++k) big_tiles += (segs[k].n + E * big_vec - 1) / (E * big_vec);
     const bool small = big_tiles < kSmallTiles;
+    bool split = false;
+    if ((job.work == kUpdate || job.work == kGeneral) && job.n_seeds >= kSplitPairs && small) {
+        uint64_t tiles = 0;
+        for (size_t k = 0; k < n_segs; ++k) tiles += (segs[k].n + 127) / 128;
+        split = tiles <= Traits<T>::SPLIT_TILES;
+    }
     const uint64_t tile_vec = small ? 32u : big_vec;
+    const uint64_t win = split ? 4 : E;  // elements of a window: a vector, or a block
     static thread_local P p;  // ~32 KB: keep it off the stack
     p.n_seeds = static_cast<uint32_t>(job.n_seeds);
     p.write_src = job.write_src ? 1u : 0u;
@@ -608,7 +778,7 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
     SEG* table = reinterpret_cast<SEG*>(p.data + p.seg_at);
 
     const uint64_t per_index = job.work == kChecksum ? E : 4;  // elements of a window or block
-    const uint64_t step = job.work == kChecksum ? 1 : E / 4;   // indices of a vector
+    const uint64_t step = job.work == kChecksum ? 1 : win / 4;  // indices of a window
     const auto high = [&](uint64_t fo) { return static_cast<uint32_t>((fo / per_index) >> 32); };
     size_t i = 0;
     uint64_t at = 0;  // elements of segs[i] already launched
@@ -623,20 +793,20 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
             const uint64_t src = segs[i].ptr + at * ES;
             const uint64_t to = dst != nullptr ? dst[i] + at * ES : src;
             SEG& g = table[count++];
-            g.head = static_cast<uint32_t>(fo % E);
+            g.head = static_cast<uint32_t>(fo % win);
             g.base = src - g.head * ES;
             g.end = g.head + n;
-            g.blk0 = static_cast<uint32_t>(fo / E * step);
+            g.blk0 = static_cast<uint32_t>(fo / win * step);
             g.tile0 = static_cast<uint32_t>(tiles);
-            // 16-byte vectors line up with element groups whose global index is a
-            // multiple of E iff the first window's address is a multiple of 16
+            // vectors line up with element groups whose global index is a multiple of E
+            // iff the first window's address is a multiple of their size
             uint64_t off = g.base;
             if constexpr (std::is_same<SEG, SegParamOut>::value) {
                 g.dst = to - g.head * ES;
                 off |= g.dst;
             }
-            g.full = (off & 15ull) == 0 ? static_cast<uint32_t>(g.end / E) : 0u;
-            const uint64_t vecs = (g.end + E - 1) / E;
+            g.full = (off & (win * ES - 1)) == 0 ? static_cast<uint32_t>(g.end / win) : 0u;
+            const uint64_t vecs = (g.end + win - 1) / win;
             tiles += (vecs + tile_vec - 1) / tile_vec;
             at += n;
             if (at == segs[i].n) {
@@ -650,6 +820,7 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
         SeedParam* sp = reinterpret_cast<SeedParam*>(p.data);
         for (int k = 0; k < job.n_seeds; ++k) sp[k] = seed_param(job.seeds[k], hi, job.coef[k]);
         for (int k = 0; k < job.n_groups; ++k) sp[job.group_end[k] - 1].ends_group = 1u;
+        if (job.work == kUpdate) sp[job.n_seeds - 1].ends_group = 1u;
         cudaError_t err;
         Job now = job;
         if (job.work == kChecksum) {
@@ -668,11 +839,11 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
         if (!small) {
             err = launch_work<T, false>(now, p);
         } else if (used > kSmallParamBytes) {
-            err = launch_work<T, true>(now, p);
+            err = split ? launch_split<T>(now, p) : launch_work<T, true>(now, p);
         } else {
             Launch<SEG, kSmallParamBytes> q;
             std::memcpy(&q, &p, offsetof(P, data) + used);
-            err = launch_work<T, true>(now, q);
+            err = split ? launch_split<T>(now, q) : launch_work<T, true>(now, q);
         }
         if (err != cudaSuccess) return err;
     }

@@ -75,6 +75,40 @@ def test_large_shape_equals_small_pieces(jb, dtype, tiles, extra, shift):
         assert torch.equal(whole.view(torch.uint8), parts.view(torch.uint8)), name
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("K", [2, 3, 8, 33, 100])
+def test_pairs_shared_out(jb, dtype, K):
+    """Tables of few tiles, whose pairs are shared out among warps, against one table over
+    all of them, which is too large for that: in place, from a source, and a replay whose
+    groups end inside a chunk of pairs. The piece lengths give groups of 16, 8 and 4 warps."""
+    seeds, q = pairs(K)
+    steps = [(seeds[a:b], q[a:b], LR, 1.0 + a) for a, b in zip([0, 1, K // 2], [1, max(K // 2, 1), K]) if b > a]
+
+    def into(t, refresh):
+        out = [torch.zeros_like(x) for x in t.tensors]
+        jb.jb_apply_updates_from(t, jb.ParamTable(out, t.flat_offsets), seeds, q, LR, DENOM, QS,
+                                 write_src=refresh)
+        if not refresh:
+            for x, o in zip(t.tensors, out):
+                x.copy_(o)
+
+    for op in (lambda t: jb.jb_apply_updates(t, seeds, q, LR, DENOM, QS), lambda t: into(t, False),
+               lambda t: into(t, True), lambda t: jb.jb_replay_updates(t, steps, QS)):
+        torch.manual_seed(K)
+        n = 400_003
+        base = torch.randn(n, device="cuda").mul_(0.02).to(dtype)
+        whole, parts = base.clone(), base.clone()
+        op(jb.ParamTable([whole], [6]))
+        cuts = np.cumsum([0, 1, 2, 3, 122, 128, 129, 5003, 152 * 128, 152 * 128 + 1, 304 * 128 + 7, 70_001, 77_000])
+        cuts = list(cuts) + [n - 70_000, n]
+        for a, b in zip(cuts, cuts[1:]):
+            mid = (a + b) // 2
+            tensors = [parts[a:b]] if b - a < 1000 else [parts[a:mid], parts[mid:b]]
+            op(jb.ParamTable(tensors, [6 + a, 6 + mid][:len(tensors)]))
+        torch.cuda.synchronize()
+        assert torch.equal(whole.view(torch.uint8), parts.view(torch.uint8))
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("vectors", [1, 31 * 32 + 1, 32 * 32, 32 * 32 + 1, 1600 * 192 - 1, 1600 * 192 + 33])
 def test_checksum_shapes(jb, dtype, vectors):
