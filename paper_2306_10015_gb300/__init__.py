@@ -65,6 +65,8 @@ _lib: Optional[ctypes.CDLL] = None
 def lib() -> ctypes.CDLL:
     """The loaded libjb.so. Raises if it has not been built."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(_LIB_PATH):
@@ -118,6 +120,9 @@ def _check(rc: int) -> None:
 def _stream(stream) -> ctypes.c_void_p:
     if stream is None:
         import torch
+        if torch.cuda.is_initialized():
+            # the current stream's handle without a Stream object around it (0.1 us, not 3)
+            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
         return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     if isinstance(stream, int):
         return ctypes.c_void_p(stream)
@@ -141,6 +146,16 @@ def seeds_array(seeds) -> np.ndarray:
     for i, s in enumerate(seeds):
         out[i] = (int(s[0]), int(s[1]), int(s[2]))
     return out
+
+
+# Host arrays go to the library as bytes objects (it copies them during the call): for the
+# few kilobytes of a call that is cheaper than asking numpy for a pointer (1 us an array).
+def _codes_array(q) -> np.ndarray:
+    return np.ascontiguousarray(np.asarray(q, dtype=np.int8))
+
+
+def _bytes(a: np.ndarray):
+    return a.tobytes() if a.size else None
 
 
 def default_flat_offsets(numels: Sequence[int], align: int = FLAT_ALIGN) -> List[int]:
@@ -207,13 +222,11 @@ def jb_perturb(table: ParamTable, seed, eps: float, stream=None, grid_ctas: int 
 def jb_apply_updates(table: ParamTable, seeds, q, lr: float, denom: float, qscale: float,
                      stream=None, grid_ctas: int = 0) -> None:
     """theta <- theta - (lr / denom) sum_k deq(q_k) z(seed_k), one pass, in place."""
-    s = seeds_array(seeds)
-    qa = np.ascontiguousarray(np.asarray(q, dtype=np.int8))
+    s, qa = seeds_array(seeds), _codes_array(q)
     if qa.shape[0] != s.shape[0]:
         raise ValueError("one byte code per seed")
     K = s.shape[0]
-    sp = ctypes.c_void_p(s.ctypes.data if K else None)
-    qp = ctypes.c_void_p(qa.ctypes.data if K else None)
+    sp, qp = _bytes(s), _bytes(qa)
     L = lib()
     if grid_ctas:
         rc = L.jb_apply_updates_with_grid(table.segments, table.n_segments, table.dtype, sp, qp, K,
@@ -230,32 +243,26 @@ def jb_apply_updates_from(src: ParamTable, dst: ParamTable, seeds, q, lr: float,
     """dst <- src - (lr / denom) sum_k deq(q_k) z(seed_k) in one pass (restore fused)."""
     if src.n_segments != dst.n_segments or src.dtype != dst.dtype:
         raise ValueError("source and destination tables differ")
-    s = seeds_array(seeds)
-    qa = np.ascontiguousarray(np.asarray(q, dtype=np.int8))
+    s, qa = seeds_array(seeds), _codes_array(q)
     if qa.shape[0] != s.shape[0]:
         raise ValueError("one byte code per seed")
-    K = s.shape[0]
     _check(lib().jb_apply_updates_from(
-        src.segments, dst.segments, src.n_segments, src.dtype,
-        ctypes.c_void_p(s.ctypes.data if K else None), ctypes.c_void_p(qa.ctypes.data if K else None),
-        K, float(lr), float(denom), float(qscale), int(bool(write_src)), _stream(stream)))
+        src.segments, dst.segments, src.n_segments, src.dtype, _bytes(s), _bytes(qa), s.shape[0],
+        float(lr), float(denom), float(qscale), int(bool(write_src)), _stream(stream)))
 
 
 def jb_replay_updates(table: ParamTable, steps, qscale: float, stream=None) -> None:
     """Apply several steps' updates in order, in place; steps = [(seeds, q, lr, denom), ...]."""
     seeds = [seeds_array(st[0]) for st in steps]
-    codes = [np.asarray(st[1], dtype=np.int8) for st in steps]
+    codes = [_codes_array(st[1]) for st in steps]
     sizes = np.array([len(x) for x in seeds], dtype=np.int32)
-    if any(len(c) != n for c, n in zip(codes, sizes)):
+    if any(len(c) != len(x) for c, x in zip(codes, seeds)):
         raise ValueError("one byte code per seed")
-    s = np.ascontiguousarray(np.concatenate(seeds) if len(seeds) else np.zeros(0, SEED_DTYPE))
-    qa = np.ascontiguousarray(np.concatenate(codes) if len(codes) else np.zeros(0, np.int8))
     lr = np.array([float(st[2]) for st in steps], dtype=np.float32)
     denom = np.array([float(st[3]) for st in steps], dtype=np.float32)
-    T = len(steps)
-    ptr = lambda a: ctypes.c_void_p(a.ctypes.data if a.size else None)
-    _check(lib().jb_replay_updates(table.segments, table.n_segments, table.dtype, ptr(s), ptr(qa),
-                                   ptr(sizes), T, ptr(lr), ptr(denom), float(qscale),
+    _check(lib().jb_replay_updates(table.segments, table.n_segments, table.dtype,
+                                   b"".join(seeds) or None, b"".join(codes) or None, _bytes(sizes),
+                                   len(steps), _bytes(lr), _bytes(denom), float(qscale),
                                    _stream(stream)))
 
 

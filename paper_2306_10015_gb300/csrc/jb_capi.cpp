@@ -59,13 +59,34 @@ int collect_segments(const jb_segment* segs, int n_segs, int dtype, std::vector<
         if (!range_fits(p, s.numel, es)) return JB_ERR_INVALID_ARG;
         out.push_back({p, s.flat_offset, s.numel});
     }
-    std::vector<Seg> by_fo(out), by_ptr(out);
-    std::sort(by_fo.begin(), by_fo.end(), [](const Seg& a, const Seg& b) { return a.fo < b.fo; });
-    for (size_t i = 1; i < by_fo.size(); ++i)
-        if (by_fo[i - 1].fo + by_fo[i - 1].n > by_fo[i].fo) return JB_ERR_INVALID_ARG;
-    std::sort(by_ptr.begin(), by_ptr.end(), [](const Seg& a, const Seg& b) { return a.ptr < b.ptr; });
-    for (size_t i = 1; i < by_ptr.size(); ++i)
-        if (by_ptr[i - 1].ptr + by_ptr[i - 1].n * es > by_ptr[i].ptr) return JB_ERR_INVALID_ARG;
+    // tables are mostly in order already; only then is no sorted copy needed
+    const auto by_fo = [](const Seg& a, const Seg& b) { return a.fo < b.fo; };
+    const auto by_ptr = [](const Seg& a, const Seg& b) { return a.ptr < b.ptr; };
+    const auto fo_overlap = [](const std::vector<Seg>& v) {
+        for (size_t i = 1; i < v.size(); ++i)
+            if (v[i - 1].fo + v[i - 1].n > v[i].fo) return true;
+        return false;
+    };
+    const auto ptr_overlap = [es](const std::vector<Seg>& v) {
+        for (size_t i = 1; i < v.size(); ++i)
+            if (v[i - 1].ptr + v[i - 1].n * es > v[i].ptr) return true;
+        return false;
+    };
+    const bool fo_sorted = std::is_sorted(out.begin(), out.end(), by_fo);
+    const bool ptr_sorted = std::is_sorted(out.begin(), out.end(), by_ptr);
+    if (fo_sorted && fo_overlap(out)) return JB_ERR_INVALID_ARG;
+    if (ptr_sorted && ptr_overlap(out)) return JB_ERR_INVALID_ARG;
+    if (!fo_sorted || !ptr_sorted) {
+        std::vector<Seg> v(out);
+        if (!fo_sorted) {
+            std::sort(v.begin(), v.end(), by_fo);
+            if (fo_overlap(v)) return JB_ERR_INVALID_ARG;
+        }
+        if (!ptr_sorted) {
+            std::sort(v.begin(), v.end(), by_ptr);
+            if (ptr_overlap(v)) return JB_ERR_INVALID_ARG;
+        }
+    }
     return JB_OK;
 }
 
@@ -74,14 +95,56 @@ jb::SeedRaw seed_raw(const jb_seed& s) {
             s.sample_id};
 }
 
-bool seed_less(const jb_seed& a, const jb_seed& b) {
-    if (a.machine_id != b.machine_id) return a.machine_id < b.machine_id;
-    if (a.step != b.step) return a.step < b.step;
-    return a.sample_id < b.sample_id;
-}
+// A pair as it is ordered: ascending (machine id, step, sample id).
+struct Pair {
+    uint64_t machine;
+    uint64_t step_sample;
+    int index;  // in the caller's arrays
+};
 
-bool seed_equal(const jb_seed& a, const jb_seed& b) {
-    return a.machine_id == b.machine_id && a.step == b.step && a.sample_id == b.sample_id;
+// Values of the byte code's magnitudes, each computed once per call.
+class Dequantizer {
+public:
+    explicit Dequantizer(float qscale) : scale_(qscale) {}
+    double operator()(int8_t q) {
+        int m = q < 0 ? -static_cast<int>(q) : static_cast<int>(q);
+        if (m > 127) m = 127;
+        if (!known_[m]) {
+            value_[m] = std::expm1(static_cast<double>(m) / scale_);
+            known_[m] = true;
+        }
+        return q < 0 ? -value_[m] : value_[m];
+    }
+
+private:
+    double scale_;
+    double value_[128];
+    bool known_[128] = {};
+};
+
+// Appends pairs [first, first + K) in canonical order with their coefficients c_k.
+int collect_pairs(const jb_seed* seeds, const int8_t* q, size_t first, int K, float lr, float denom,
+                  Dequantizer& deq, std::vector<jb::SeedRaw>& raw, std::vector<float>& coef) {
+    std::vector<Pair> order(static_cast<size_t>(K));
+    for (int k = 0; k < K; ++k) {
+        const jb_seed& s = seeds[first + k];
+        order[k] = {s.machine_id, (static_cast<uint64_t>(s.step) << 32) | s.sample_id, k};
+    }
+    std::sort(order.begin(), order.end(), [](const Pair& a, const Pair& b) {
+        return a.machine != b.machine ? a.machine < b.machine : a.step_sample < b.step_sample;
+    });
+    for (int k = 1; k < K; ++k)
+        if (order[k - 1].machine == order[k].machine && order[k - 1].step_sample == order[k].step_sample)
+            return JB_ERR_DUPLICATE_SEED;
+    for (const Pair& o : order) {
+        const size_t i = first + static_cast<size_t>(o.index);
+        const double c = -static_cast<double>(lr) * deq(q[i]) / static_cast<double>(denom);
+        const float cf = static_cast<float>(c);
+        if (!std::isfinite(cf)) return JB_ERR_RANGE;
+        raw.push_back(seed_raw(seeds[i]));
+        coef.push_back(cf);
+    }
+    return JB_OK;
 }
 
 double dequantize(int8_t q, double qscale) {
@@ -126,24 +189,13 @@ int update_impl(const jb_segment* segs, int n_segs, int dtype, const jb_seed* se
     if (K > jb::kMaxSeedsPerLaunch) return JB_ERR_TOO_MANY_SEEDS;
     if (K == 0) return JB_OK;
 
-    // Canonical order: ascending (machine id, step, sample id).
-    std::vector<int> order(static_cast<size_t>(K));
-    for (int k = 0; k < K; ++k) order[k] = k;
-    std::stable_sort(order.begin(), order.end(),
-                     [&](int a, int b) { return seed_less(seeds[a], seeds[b]); });
-    for (int k = 1; k < K; ++k)
-        if (seed_equal(seeds[order[k - 1]], seeds[order[k]])) return JB_ERR_DUPLICATE_SEED;
-
-    std::vector<jb::SeedRaw> raw(static_cast<size_t>(K));
-    std::vector<float> coef(static_cast<size_t>(K));
-    for (int k = 0; k < K; ++k) {
-        const int i = order[k];
-        const double c = -static_cast<double>(lr) * dequantize(q[i], static_cast<double>(qscale)) /
-                         static_cast<double>(denom);
-        coef[k] = static_cast<float>(c);
-        if (!std::isfinite(coef[k])) return JB_ERR_RANGE;
-        raw[k] = seed_raw(seeds[i]);
-    }
+    std::vector<jb::SeedRaw> raw;
+    std::vector<float> coef;
+    raw.reserve(static_cast<size_t>(K));
+    coef.reserve(static_cast<size_t>(K));
+    Dequantizer deq(qscale);
+    rc = collect_pairs(seeds, q, 0, K, lr, denom, deq, raw, coef);
+    if (rc != JB_OK) return rc;
     if (v.empty()) return JB_OK;
     jb::Job job{jb::kUpdate, dtype, raw.data(), coef.data(), K, nullptr, 0, false, grid_ctas, stream, nullptr};
     return cuda_status(jb::enqueue(job, v.data(), nullptr, v.size()));
@@ -212,28 +264,16 @@ int general_impl(const jb_segment* segs, const jb_segment* dsts, int n_segs, int
     if (total > 0 && (seeds == nullptr || q == nullptr)) return JB_ERR_INVALID_ARG;
 
     // every group in canonical order, with its coefficients
-    std::vector<jb::SeedRaw> raw(static_cast<size_t>(total));
-    std::vector<float> coef(static_cast<size_t>(total));
+    std::vector<jb::SeedRaw> raw;
+    std::vector<float> coef;
+    raw.reserve(static_cast<size_t>(total));
+    coef.reserve(static_cast<size_t>(total));
+    Dequantizer deq(qscale);
     std::vector<int> sizes;
-    long long base = 0;
     for (int g = 0; g < n_groups; ++g) {
         const int K = group_sizes[g];
-        std::vector<int> order(static_cast<size_t>(K));
-        for (int k = 0; k < K; ++k) order[k] = static_cast<int>(base) + k;
-        std::stable_sort(order.begin(), order.end(),
-                         [&](int a, int b) { return seed_less(seeds[a], seeds[b]); });
-        for (int k = 1; k < K; ++k)
-            if (seed_equal(seeds[order[k - 1]], seeds[order[k]])) return JB_ERR_DUPLICATE_SEED;
-        for (int k = 0; k < K; ++k) {
-            const int i = order[k];
-            const double c = -static_cast<double>(lr[g]) * dequantize(q[i], static_cast<double>(qscale)) /
-                             static_cast<double>(denom[g]);
-            const float cf = static_cast<float>(c);
-            if (!std::isfinite(cf)) return JB_ERR_RANGE;
-            raw[static_cast<size_t>(base + k)] = seed_raw(seeds[i]);
-            coef[static_cast<size_t>(base + k)] = cf;
-        }
-        base += K;
+        rc = collect_pairs(seeds, q, raw.size(), K, lr[g], denom[g], deq, raw, coef);
+        if (rc != JB_OK) return rc;
         if (K > 0) sizes.push_back(K);  // an empty group changes nothing
     }
     if (v.empty()) return JB_OK;
@@ -365,7 +405,8 @@ int perturb_q4_impl(const jb_q4_segment* segs, int n_segs, jb_seed seed, float e
         idx.push_back({g.flat_offset, g.flat_offset + g.numel});
     }
     for (auto* list : {&mem, &idx}) {
-        std::sort(list->begin(), list->end(), [](const Iv& x, const Iv& y) { return x.a < y.a; });
+        const auto before = [](const Iv& x, const Iv& y) { return x.a < y.a; };
+        if (!std::is_sorted(list->begin(), list->end(), before)) std::sort(list->begin(), list->end(), before);
         for (size_t i = 1; i < list->size(); ++i)
             if ((*list)[i - 1].b > (*list)[i].a) return JB_ERR_INVALID_ARG;
     }
