@@ -74,8 +74,11 @@ struct SegParam {
     uint64_t end;    // elements of the segment are [head, end) of its windows
     uint32_t blk0;   // low word of the Philox block index of the first window (checksum: its own)
     uint32_t tile0;  // first tile
-    uint32_t head;   // elements of the first window before the segment (0 .. E - 1)
-    uint32_t full;   // vectors [head ? 1 : 0, full) take 16-byte accesses; 0: none does
+    uint8_t head;    // elements of the first window before the segment (0 .. E - 1)
+    uint8_t lo;      // vectors [lo, full) are read and written whole; the others go element
+    uint8_t load;    //   by element. Alignment of their addresses, 2 to 16 bytes: of the
+    uint8_t store;   //   source, and of where the result goes
+    uint32_t full;
 };
 
 struct SegParamOut : SegParam {

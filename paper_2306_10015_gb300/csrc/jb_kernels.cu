@@ -53,6 +53,8 @@ namespace {
 //                    bf16 2 x 512: 2696 (2 x 768: 2755, 3 x 512: 2782)
 //   checksum         fp32 6 x 512: 152.0 (8 x 512: 153.4, 4 x 512: 157), bf16 79.9 (81.1, 83.2);
 //                    1.3B bf16 359 either way: 7.3 TB/s
+//   one pair that writes source and destination, fp32 (memory alone: 474): 16 warps per SM
+//                    4 x 512: 481; more of them in flight cost bandwidth (4 x 1024: 525)
 //   one pair         fp32 4 x 1024: 319 (4 x 768: 328, 4 x 512: 329; HBM alone: 316)
 //                    bf16 4 x 1024: 289 (4 x 768: 293, 4 x 512: 302, 8 x 768: 284)
 // Small tables take one vector per thread in every kernel, and their launch fewer
@@ -60,9 +62,10 @@ namespace {
 // counts is that all 608 have some. The line lies where the large shape gives most of its
 // 16 warps per SM a tile (K = 32 update, us, one vector / large shape; fp32 512K elements
 // 27 / 29, 1M 43 / 40, 2M 84 / 77; bf16 512K 25 / 33, 1M 43 / 47, 1.5M 62 / 59, 3M 111 / 103).
-template <int V_, int THREADS_, int UNROLL_>
+template <int V_, int THREADS_, int UNROLL_, int CTAS_ = 0>
 struct Shape {
     static constexpr int V = V_, THREADS = THREADS_, UNROLL = UNROLL_;
+    static constexpr int CTAS = CTAS_;  // most CTAs per SM (0: as many as fit)
 };
 
 constexpr uint64_t kSmallTiles = 1600;  // tiles of the large shape
@@ -76,6 +79,7 @@ struct Traits<float> {
     using Update = Shape<5, 512, 2>;
     using General = Shape<4, 512, 2>;
     using Pair = Shape<4, 1024, 1>;
+    using Refresh = Shape<4, 512, 1, 1>;
     using Sum = Shape<6, 512, 1>;
     using Small = Shape<1, 512, 2>;
 };
@@ -86,6 +90,7 @@ struct Traits<__nv_bfloat16> {
     using Update = Shape<3, 512, 2>;
     using General = Shape<2, 512, 2>;
     using Pair = Shape<4, 1024, 1>;
+    using Refresh = Pair;
     using Sum = Shape<6, 512, 1>;
     using Small = Shape<1, 512, 2>;
 };
@@ -120,6 +125,49 @@ __device__ __forceinline__ uint4 pack(const float2 (&x)[2][2]) {
 
 __device__ __forceinline__ uint4 load_vec(uint64_t a) { return __ldcs(reinterpret_cast<const uint4*>(a)); }
 __device__ __forceinline__ void store_vec(uint64_t a, uint4 w) { __stcs(reinterpret_cast<uint4*>(a), w); }
+
+// A whole vector at an address that is a multiple of `align` = 8, 4 or 2 bytes only: two
+// or four accesses, or, on an odd multiple of 2, the five words that it lies in (the
+// caller sees to it that they belong to the segment), of which the two at the ends are
+// written by halves. A tensor off the 16-byte grid of its flat offset takes these, in
+// kernels of their own (OFF; in the common ones the choice costs registers). One
+// perturbation of 2^28 elements, against element by element: bf16 295 us at 8 bytes, 307
+// at 4, 415 at 2 (541 to 615 before; 289 on the grid), fp32 343 and 360 (427; 318).
+__device__ __forceinline__ uint4 load_off_grid(uint64_t a, uint32_t align) {
+    uint4 w;
+    if (align == 8u) {
+        const uint2 p = __ldcs(reinterpret_cast<const uint2*>(a)), q = __ldcs(reinterpret_cast<const uint2*>(a) + 1);
+        w = make_uint4(p.x, p.y, q.x, q.y);
+    } else if (align == 4u) {
+        const uint32_t* p = reinterpret_cast<const uint32_t*>(a);
+        w = make_uint4(__ldcs(p), __ldcs(p + 1), __ldcs(p + 2), __ldcs(p + 3));
+    } else {
+        const uint32_t* p = reinterpret_cast<const uint32_t*>(a - 2);
+        const uint32_t q[5] = {__ldcs(p), __ldcs(p + 1), __ldcs(p + 2), __ldcs(p + 3), __ldcs(p + 4)};
+        w = make_uint4(__funnelshift_r(q[0], q[1], 16), __funnelshift_r(q[1], q[2], 16),
+                       __funnelshift_r(q[2], q[3], 16), __funnelshift_r(q[3], q[4], 16));
+    }
+    return w;
+}
+__device__ __forceinline__ void store_off_grid(uint64_t a, uint32_t align, uint4 w) {
+    if (align == 8u) {
+        __stcs(reinterpret_cast<uint2*>(a), make_uint2(w.x, w.y));
+        __stcs(reinterpret_cast<uint2*>(a) + 1, make_uint2(w.z, w.w));
+    } else if (align == 4u) {
+        uint32_t* p = reinterpret_cast<uint32_t*>(a);
+        __stcs(p, w.x);
+        __stcs(p + 1, w.y);
+        __stcs(p + 2, w.z);
+        __stcs(p + 3, w.w);
+    } else {
+        *reinterpret_cast<uint16_t*>(a) = static_cast<uint16_t>(w.x);
+        uint32_t* p = reinterpret_cast<uint32_t*>(a + 2);
+        __stcs(p, __funnelshift_r(w.x, w.y, 16));
+        __stcs(p + 1, __funnelshift_r(w.y, w.z, 16));
+        __stcs(p + 2, __funnelshift_r(w.z, w.w, 16));
+        *reinterpret_cast<uint16_t*>(a + 14) = static_cast<uint16_t>(w.w >> 16);
+    }
+}
 
 // Elements [first, last) of the window at address a (the others read as zero bits).
 template <typename T>
@@ -185,8 +233,8 @@ enum Store { kInPlace, kToDst, kNowhere };
 // another go to different SMs, so that a few tiles occupy as many SMs. Which warp
 // handles a tile never changes a result: every element's value depends only on its own
 // stored value, its global index and the seeds. Vectors that are partial (the ends of a
-// segment), or whose segment lies off the 16-byte grid, go element by element.
-template <typename T, typename S, Store TO, typename P, typename Op>
+// segment) go element by element. OFF: segments may lie off the 16-byte grid.
+template <typename T, typename S, Store TO, bool OFF, typename P, typename Op>
 __device__ __forceinline__ void visit_tiles(const P& p, bool also_src, Op&& op) {
     constexpr int E = Traits<T>::E, V = S::V;
     constexpr uint32_t B = TO == kNowhere ? 1 : E / 4, kTileVec = 32u * V;
@@ -203,7 +251,8 @@ __device__ __forceinline__ void visit_tiles(const P& p, bool also_src, Op&& op) 
             const auto& g = seg_at(p, s);
             const uint32_t next = seg_at(p, s + 1).tile0;
             const uint32_t stop = next < t_end ? next : t_end;
-            const uint32_t v_lo = g.head != 0u ? 1u : 0u, v_hi = g.full;
+            const uint32_t v_lo = g.lo, v_hi = g.full;
+            const uint32_t load_align = OFF ? g.load : 16u, store_align = OFF ? g.store : 16u;
             uint32_t v = (t - g.tile0) * kTileVec;  // first vector of the tile
             uint64_t src = g.base + 16ull * (v + lane);
             uint64_t dst = dst_of(g) + 16ull * (v + lane);
@@ -212,14 +261,17 @@ __device__ __forceinline__ void visit_tiles(const P& p, bool also_src, Op&& op) 
             for (; t < stop; ++t) {
                 const bool fast = v >= v_lo && v + kTileVec <= v_hi;  // the same for every lane
                 uint4 x[V];
-                if (fast) {
+                if (fast && load_align == 16u) {
 #pragma unroll
                     for (int j = 0; j < V; ++j) x[j] = load_vec(src + 512ull * j);
+                } else if (fast) {
+#pragma unroll
+                    for (int j = 0; j < V; ++j) x[j] = load_off_grid(src + 512ull * j, load_align);
                 } else {
 #pragma unroll
                     for (int j = 0; j < V; ++j) {
                         const uint32_t vj = v + lane + 32u * j;
-                        if (vj >= v_lo && vj < v_hi) {
+                        if (vj >= v_lo && vj < v_hi && load_align == 16u) {
                             x[j] = load_vec(src + 512ull * j);
                         } else {
                             const uint64_t e0 = static_cast<uint64_t>(vj) * E;
@@ -237,17 +289,29 @@ __device__ __forceinline__ void visit_tiles(const P& p, bool also_src, Op&& op) 
                 constexpr bool TO_DST = TO == kToDst;
                 const uint64_t out = TO_DST ? dst : src;
                 if constexpr (TO == kNowhere) {
-                } else if (fast) {
+                } else if (fast && store_align == 16u) {
 #pragma unroll
                     for (int j = 0; j < V; ++j) {
                         store_vec(out + 512ull * j, x[j]);
-                        if (TO_DST && also_src) store_vec(src + 512ull * j, x[j]);
+                        if (TO_DST && also_src) {
+                            if (load_align == 16u) store_vec(src + 512ull * j, x[j]);
+                            else store_off_grid(src + 512ull * j, load_align, x[j]);
+                        }
+                    }
+                } else if (fast) {
+#pragma unroll
+                    for (int j = 0; j < V; ++j) {
+                        store_off_grid(out + 512ull * j, store_align, x[j]);
+                        if (TO_DST && also_src) {
+                            if (load_align == 16u) store_vec(src + 512ull * j, x[j]);
+                            else store_off_grid(src + 512ull * j, load_align, x[j]);
+                        }
                     }
                 } else {
 #pragma unroll
                     for (int j = 0; j < V; ++j) {
                         const uint32_t vj = v + lane + 32u * j;
-                        if (vj >= v_lo && vj < v_hi) {
+                        if (vj >= v_lo && vj < v_hi && load_align == 16u && store_align == 16u) {
                             store_vec(out + 512ull * j, x[j]);
                             if (TO_DST && also_src) store_vec(src + 512ull * j, x[j]);
                         } else {
@@ -343,9 +407,9 @@ __device__ __forceinline__ void update_tile(const P& p, uint4 (&x)[S::V], uint32
     }
 }
 
-template <typename T, typename S, typename P>
+template <typename T, typename S, bool OFF, typename P>
 __global__ void __launch_bounds__(S::THREADS) seeded_kernel(const __grid_constant__ P p) {
-    visit_tiles<T, S, kInPlace>(p, false, [&](uint4 (&x)[S::V], uint32_t blk) {
+    visit_tiles<T, S, kInPlace, OFF>(p, false, [&](uint4 (&x)[S::V], uint32_t blk) {
         update_tile<T, S, false>(p, x, blk);
     });
 }
@@ -387,10 +451,10 @@ __device__ __forceinline__ void one_seed_tile(const P& p, uint4 (&x)[V], uint32_
 
 enum OneSeed { kPerturbInPlace = 0, kAddInPlace = 1, kAddToDst = 2 };
 
-template <typename T, typename S, int MODE, typename P>
+template <typename T, typename S, int MODE, bool OFF, typename P>
 __global__ void __launch_bounds__(S::THREADS) one_seed_kernel(const __grid_constant__ P p) {
     constexpr bool TO_DST = MODE == kAddToDst;
-    visit_tiles<T, S, TO_DST ? kToDst : kInPlace>(p, TO_DST && p.write_src != 0u, [&](uint4 (&x)[S::V], uint32_t blk) {
+    visit_tiles<T, S, TO_DST ? kToDst : kInPlace, OFF>(p, TO_DST && p.write_src != 0u, [&](uint4 (&x)[S::V], uint32_t blk) {
         one_seed_tile<T, S::V, MODE == kPerturbInPlace>(p, x, blk);
     });
 }
@@ -398,9 +462,9 @@ __global__ void __launch_bounds__(S::THREADS) one_seed_kernel(const __grid_const
 // The generalised update: source -> destination (optionally also back to the
 // source), seeds applied in groups with a rounding to the storage type after each
 // group, exactly as successive in-place updates would round.
-template <typename T, typename S, typename P>
+template <typename T, typename S, bool OFF, typename P>
 __global__ void __launch_bounds__(S::THREADS) general_update_kernel(const __grid_constant__ P p) {
-    visit_tiles<T, S, kToDst>(p, p.write_src != 0u, [&](uint4 (&x)[S::V], uint32_t blk) {
+    visit_tiles<T, S, kToDst, OFF>(p, p.write_src != 0u, [&](uint4 (&x)[S::V], uint32_t blk) {
         update_tile<T, S, true>(p, x, blk);
     });
 }
@@ -509,7 +573,7 @@ __global__ void __launch_bounds__(kSplitThreads) split_update_kernel(const __gri
         const uint64_t e0 = 4ull * v;
         const int first = v == 0u ? static_cast<int>(g.head) : 0;
         const int last = e0 >= g.end ? 0 : (g.end - e0 < 4 ? static_cast<int>(g.end - e0) : 4);
-        const bool full = v >= (g.head != 0u ? 1u : 0u) && v < g.full;
+        const bool full = v >= g.lo && v < g.full;
         const uint64_t src = g.base + 4ull * ES * v;
         float x[4];
         float2 even = make_float2(0.0f, 0.0f), odd = even;
@@ -576,11 +640,11 @@ __device__ __forceinline__ uint64_t window_hash(uint64_t win, uint4 w) {
 
 // blk0 of the segments is the low word of the index of the first window, p.window_hi
 // the high word of all. One CTA alone stores its sum, which saves the clearing of *out.
-template <typename T, typename S, typename P>
+template <typename T, typename S, bool OFF, typename P>
 __global__ void __launch_bounds__(S::THREADS) checksum_kernel(const __grid_constant__ P p,
                                                              unsigned long long* out) {
     uint64_t sum = 0;
-    visit_tiles<T, S, kNowhere>(p, false, [&](uint4 (&x)[S::V], uint32_t win, uint32_t present) {
+    visit_tiles<T, S, kNowhere, OFF>(p, false, [&](uint4 (&x)[S::V], uint32_t win, uint32_t present) {
 #pragma unroll
         for (int j = 0; j < S::V; ++j) {
             const uint64_t w = (static_cast<uint64_t>(p.window_hi) << 32) | (win + 32u * j);
@@ -660,7 +724,8 @@ __global__ void debug_box_muller_kernel(const uint32_t* words, uint64_t n, float
     }
 }
 
-// Persistent grid: SM count x resident CTAs per SM, cached per device and kernel.
+// Persistent grid: SM count x resident CTAs per SM (`most` at most, 0: no limit), cached
+// per device and kernel.
 constexpr int kMaxDevices = 64;
 
 struct GridCache {
@@ -668,7 +733,7 @@ struct GridCache {
 };
 
 template <typename K>
-cudaError_t persistent_grid(K kernel, int threads, GridCache& cache, int* grid) {
+cudaError_t persistent_grid(K kernel, int threads, int most, GridCache& cache, int* grid) {
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
@@ -684,6 +749,7 @@ cudaError_t persistent_grid(K kernel, int threads, GridCache& cache, int* grid) 
     if (err != cudaSuccess) return err;
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
     if (err != cudaSuccess) return err;
+    if (most > 0 && per_sm > most) per_sm = most;
     *grid = sms * (per_sm > 0 ? per_sm : 1);
     if (dev < kMaxDevices) cache.ctas[dev].store(*grid, std::memory_order_relaxed);
     return cudaSuccess;
@@ -696,7 +762,7 @@ template <typename S, typename P, typename K, typename... More>
 cudaError_t launch(K kernel, GridCache& cache, P& p, int grid_ctas, cudaStream_t stream, More... more) {
     int grid = grid_ctas;
     if (grid <= 0) {
-        cudaError_t err = persistent_grid(kernel, S::THREADS, cache, &grid);
+        cudaError_t err = persistent_grid(kernel, S::THREADS, S::CTAS, cache, &grid);
         if (err != cudaSuccess) return err;
     }
     const uint64_t warps = static_cast<uint64_t>(grid) * (S::THREADS / 32);
@@ -715,7 +781,7 @@ cudaError_t launch_split(const Job& job, P& p) {
     static GridCache cache;
     auto kernel = split_update_kernel<T, std::is_same<typename P::Seg, SegParamOut>::value, P>;
     int sms = 0;
-    cudaError_t err = persistent_grid(kernel, kSplitThreads, cache, &sms);
+    cudaError_t err = persistent_grid(kernel, kSplitThreads, 1, cache, &sms);
     if (err != cudaSuccess) return err;
     const uint32_t ctas = static_cast<uint32_t>(job.grid_ctas > 0 ? job.grid_ctas : sms);
     p.span = p.n_tiles <= ctas ? 16u : p.n_tiles <= 2u * ctas ? 8u : 4u;
@@ -726,7 +792,7 @@ cudaError_t launch_split(const Job& job, P& p) {
     return cudaGetLastError();
 }
 
-template <typename T, bool SMALL, typename P>
+template <typename T, bool SMALL, bool OFF, typename P>
 cudaError_t launch_work(const Job& job, P& p) {
     static GridCache caches[4];
     using C = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::Sum>;
@@ -735,17 +801,20 @@ cudaError_t launch_work(const Job& job, P& p) {
     using S = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::Pair>;
     const int ctas = job.grid_ctas;
     if constexpr (std::is_same<typename P::Seg, SegParamOut>::value) {
+        using R = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::Refresh>;
+        if (p.n_seeds == 1 && p.write_src != 0u)
+            return launch<R>(one_seed_kernel<T, R, kAddToDst, OFF, P>, caches[2], p, ctas, job.stream);
         if (p.n_seeds == 1)
-            return launch<S>(one_seed_kernel<T, S, kAddToDst, P>, caches[0], p, ctas, job.stream);
-        return launch<G>(general_update_kernel<T, G, P>, caches[1], p, ctas, job.stream);
+            return launch<S>(one_seed_kernel<T, S, kAddToDst, OFF, P>, caches[0], p, ctas, job.stream);
+        return launch<G>(general_update_kernel<T, G, OFF, P>, caches[1], p, ctas, job.stream);
     } else {
         if (job.work == kChecksum)
-            return launch<C>(checksum_kernel<T, C, P>, caches[3], p, ctas, job.stream, job.sum);
+            return launch<C>(checksum_kernel<T, C, OFF, P>, caches[3], p, ctas, job.stream, job.sum);
         if (job.work == kPerturb)
-            return launch<S>(one_seed_kernel<T, S, kPerturbInPlace, P>, caches[0], p, ctas, job.stream);
+            return launch<S>(one_seed_kernel<T, S, kPerturbInPlace, OFF, P>, caches[0], p, ctas, job.stream);
         if (p.n_seeds == 1)
-            return launch<S>(one_seed_kernel<T, S, kAddInPlace, P>, caches[1], p, ctas, job.stream);
-        return launch<U>(seeded_kernel<T, U, P>, caches[2], p, ctas, job.stream);
+            return launch<S>(one_seed_kernel<T, S, kAddInPlace, OFF, P>, caches[1], p, ctas, job.stream);
+        return launch<U>(seeded_kernel<T, U, OFF, P>, caches[2], p, ctas, job.stream);
     }
 }
 
@@ -756,7 +825,7 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
     using P = Launch<SEG, kParamBytes>;
     constexpr uint64_t E = Traits<T>::E, ES = sizeof(T);
     const uint64_t big_vec = 32ull * (job.work == kChecksum  ? Traits<T>::Sum::V
-                                      : job.n_seeds == 1     ? Traits<T>::Pair::V
+                                      : job.n_seeds == 1     ? Traits<T>::Pair::V  // = Refresh::V
                                       : job.work == kGeneral ? Traits<T>::General::V
                                                              : Traits<T>::Update::V);
     uint64_t big_tiles = 0;
@@ -787,25 +856,40 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
         const uint32_t hi = high(segs[i].fo + at);
         size_t count = 0;
         uint64_t tiles = 0;
+        bool off_grid = false;
         while (i < n_segs && count < room && high(segs[i].fo + at) == hi && tiles < (1ull << 30)) {
             const uint64_t fo = segs[i].fo + at;
             const uint64_t n = std::min(segs[i].n - at, kPieceElems - fo % kPieceElems);
             const uint64_t src = segs[i].ptr + at * ES;
             const uint64_t to = dst != nullptr ? dst[i] + at * ES : src;
             SEG& g = table[count++];
-            g.head = static_cast<uint32_t>(fo % win);
-            g.base = src - g.head * ES;
-            g.end = g.head + n;
+            const uint64_t head = fo % win;
+            g.head = static_cast<uint8_t>(head);
+            g.base = src - head * ES;
+            g.end = head + n;
             g.blk0 = static_cast<uint32_t>(fo / win * step);
             g.tile0 = static_cast<uint32_t>(tiles);
-            // vectors line up with element groups whose global index is a multiple of E
-            // iff the first window's address is a multiple of their size
-            uint64_t off = g.base;
+            // a vector's address is a multiple of its size iff the segment's is where its
+            // flat offset is; otherwise vectors are put together from smaller accesses
+            uint64_t where = g.base;
             if constexpr (std::is_same<SEG, SegParamOut>::value) {
-                g.dst = to - g.head * ES;
-                off |= g.dst;
+                g.dst = to - head * ES;
+                where = g.dst;
             }
-            g.full = (off & (win * ES - 1)) == 0 ? static_cast<uint32_t>(g.end / win) : 0u;
+            const uint64_t size = win * ES;
+            const auto align = [size](uint64_t a) { return static_cast<uint8_t>(std::min(size, (a | size) & (~(a | size) + 1))); };
+            g.load = align(g.base);
+            g.store = align(where);
+            if (g.load != size || g.store != size) off_grid = true;
+            g.lo = head != 0 ? 1 : 0;
+            g.full = static_cast<uint32_t>(g.end / win);
+            if (split) {
+                if (g.load != size || g.store != size) g.full = 0;  // element by element
+            } else if (g.load == 2 || g.store == 2) {
+                // reads and writes reach two bytes past a vector on both sides
+                g.lo += 1;
+                g.full = g.full > 1 ? g.full - 1 : 0;
+            }
             const uint64_t vecs = (g.end + win - 1) / win;
             tiles += (vecs + tile_vec - 1) / tile_vec;
             at += n;
@@ -836,14 +920,18 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
             }
         }
         const size_t used = p.seg_at + (count + 1) * sizeof(SEG);
-        if (!small) {
-            err = launch_work<T, false>(now, p);
-        } else if (used > kSmallParamBytes) {
-            err = split ? launch_split<T>(now, p) : launch_work<T, true>(now, p);
+        if (split || (small && !off_grid)) {
+            if (used > kSmallParamBytes) {
+                err = split ? launch_split<T>(now, p) : launch_work<T, true, false>(now, p);
+            } else {
+                Launch<SEG, kSmallParamBytes> q;
+                std::memcpy(&q, &p, offsetof(P, data) + used);
+                err = split ? launch_split<T>(now, q) : launch_work<T, true, false>(now, q);
+            }
+        } else if (small) {
+            err = launch_work<T, true, true>(now, p);
         } else {
-            Launch<SEG, kSmallParamBytes> q;
-            std::memcpy(&q, &p, offsetof(P, data) + used);
-            err = split ? launch_split<T>(now, q) : launch_work<T, true>(now, q);
+            err = off_grid ? launch_work<T, false, true>(now, p) : launch_work<T, false, false>(now, p);
         }
         if (err != cudaSuccess) return err;
     }
@@ -876,7 +964,7 @@ cudaError_t launch_debug_philox_fold(SeedRaw seed, uint64_t first, uint64_t n, u
     cudaError_t err = cudaMemsetAsync(out, 0, sizeof(uint32_t), s);
     if (err != cudaSuccess || n == 0) return err;
     int full_grid = 0;
-    err = persistent_grid(debug_philox_fold_kernel, kThreads, cache, &full_grid);
+    err = persistent_grid(debug_philox_fold_kernel, kThreads, 0, cache, &full_grid);
     if (err != cudaSuccess) return err;
     while (n > 0) {  // one launch per high word of the block index
         const uint64_t m = std::min<uint64_t>(n, (1ull << 32) - (first & 0xFFFFFFFFull));

@@ -76,6 +76,57 @@ def test_large_shape_equals_small_pieces(jb, dtype, tiles, extra, shift):
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n", [7, 33, 4099, 400_003, 1_700_021])
+def test_off_grid_equals_aligned(jb, dtype, n):
+    """Tensors that start at every element of the 16-byte grid of their flat offsets (8, 4
+    and 2 byte alignment, a head or none) against the aligned one; what lies around them
+    stays as it was. From a source and into a destination of other alignments too."""
+    torch.manual_seed(n)
+    values = torch.randn(n, device="cuda").mul_(0.02).to(dtype)
+    per = 16 // values.element_size()
+
+    def placed(shift, fill=7.0):
+        buf = torch.full((n + 64,), fill, device="cuda", dtype=dtype)
+        buf[16 + shift:16 + shift + n] = values
+        return buf, buf[16 + shift:16 + shift + n]
+
+    def check(buf, part, want, what):
+        assert torch.equal(part.view(torch.uint8), want.view(torch.uint8)), what
+        start = part.storage_offset()
+        assert bool((buf[:start] == 7.0).all()) and bool((buf[start + n:] == 7.0).all()), what
+
+    ops = operations(jb)
+    for fo in (8, 11):
+        wants = {}
+        for name, op in ops.items():
+            buf, part = placed(fo % per)  # on the grid
+            op(jb.ParamTable([part], [fo]))
+            wants[name] = part.clone()
+        total = torch.zeros(1, dtype=torch.int64, device="cuda")
+        jb.jb_checksum(jb.ParamTable([placed(fo % per)[1]], [fo]), total)
+        for shift in range(per):
+            for name, op in ops.items():
+                if name.startswith("from"):
+                    continue
+                buf, part = placed(shift)
+                op(jb.ParamTable([part], [fo]))
+                check(buf, part, wants[name], (fo, shift, name))
+            buf, part = placed(shift)
+            got = torch.zeros(1, dtype=torch.int64, device="cuda")
+            jb.jb_checksum(jb.ParamTable([part], [fo]), got)
+            assert int(got.item()) == int(total.item())
+            for K in (1, 4):
+                for to in (0, 1, 2, per // 2):
+                    src, s = placed(shift)
+                    dst, d = placed(to)
+                    d.zero_()
+                    jb.jb_apply_updates_from(jb.ParamTable([s], [fo]), jb.ParamTable([d], [fo]), *pairs(K), LR,
+                                             DENOM, QS, write_src=(to == 1))
+                    check(dst, d, wants[f"from K={K}"], (fo, shift, to, K))
+                    check(src, s, wants[f"from K={K}"] if to == 1 else values, (fo, shift, to, K))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("K", [2, 3, 8, 33, 100])
 def test_pairs_shared_out(jb, dtype, K):
     """Tables of few tiles, whose pairs are shared out among warps, against one table over
