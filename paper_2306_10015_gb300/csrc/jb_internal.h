@@ -69,6 +69,21 @@ __host__ __device__ inline SeedParam seed_param(const SeedRaw& s, uint32_t block
     return r;
 }
 
+// A pair with the round keys of rounds 3 .. 10, which the kernels otherwise add up for
+// every pair and tile.
+struct KeyedParam : SeedParam {
+    uint32_t key[16];
+};
+
+inline void set_pair(SeedParam& to, const SeedParam& s) { to = s; }
+inline void set_pair(KeyedParam& to, const SeedParam& s) {
+    static_cast<SeedParam&>(to) = s;
+    for (uint32_t r = 0; r < 8; ++r) {
+        to.key[2 * r] = s.k0 + r * kPhiloxW0;
+        to.key[2 * r + 1] = s.k1 + r * kPhiloxW1;
+    }
+}
+
 struct SegParam {
     uint64_t base;   // device address of the segment's first window (its element `head` is element 0)
     uint64_t end;    // elements of the segment are [head, end) of its windows
@@ -85,9 +100,10 @@ struct SegParamOut : SegParam {
     uint64_t dst;    // destination address of the first window
 };
 
-template <typename SEG, int BYTES>
+template <typename SEG, typename PAIR, int BYTES>
 struct Launch {
     using Seg = SEG;
+    using Pair = PAIR;
     static constexpr int kBytes = BYTES;
     uint32_t n_seeds;
     uint32_t n_segs;
@@ -103,7 +119,7 @@ constexpr int kParamBytes = 32704;
 // Small launches: the parameters are copied for each launch (an empty kernel: 10.8 us
 // from call to end with 32 KB of them, 9.0 us with 4 KB).
 constexpr int kSmallParamBytes = 4064;
-static_assert(sizeof(Launch<SegParam, kParamBytes>) <= 32764, "launch exceeds the parameter space");
+static_assert(sizeof(Launch<SegParam, SeedParam, kParamBytes>) <= 32764, "launch exceeds the parameter space");
 
 // A checked segment: element i at ptr + i sizeof(T) has global index fo + i.
 struct Seg {

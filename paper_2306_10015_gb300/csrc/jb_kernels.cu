@@ -198,8 +198,8 @@ __device__ __forceinline__ void store_part(uint64_t a, int first, int last, uint
 }
 
 template <typename P>
-__device__ __forceinline__ const SeedParam& seed_at(const P& p, uint32_t k) {
-    return reinterpret_cast<const SeedParam*>(p.data)[k];
+__device__ __forceinline__ const typename P::Pair& seed_at(const P& p, uint32_t k) {
+    return reinterpret_cast<const typename P::Pair*>(p.data)[k];
 }
 template <typename P>
 __device__ __forceinline__ const typename P::Seg& seg_at(const P& p, uint32_t s) {
@@ -380,7 +380,7 @@ __device__ __forceinline__ void update_tile(const P& p, uint4 (&x)[S::V], uint32
 #pragma unroll
     for (int i = 0; i < NB; ++i) w[i] = philox_block(seed_at(p, 0), bc[i]);
     auto pair = [&](uint32_t k, auto more) {
-        const SeedParam& sd = seed_at(p, k);
+        const auto& sd = seed_at(p, k);
         const float2 c = splat(sd.coef);
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
@@ -800,7 +800,12 @@ cudaError_t launch_work(const Job& job, P& p) {
     using G = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::General>;
     using S = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::Pair>;
     const int ctas = job.grid_ctas;
-    if constexpr (std::is_same<typename P::Seg, SegParamOut>::value) {
+    if constexpr (std::is_same<typename P::Pair, KeyedParam>::value) {
+        if constexpr (std::is_same<typename P::Seg, SegParamOut>::value)
+            return launch<G>(general_update_kernel<T, G, OFF, P>, caches[0], p, ctas, job.stream);
+        else
+            return launch<U>(seeded_kernel<T, U, OFF, P>, caches[0], p, ctas, job.stream);
+    } else if constexpr (std::is_same<typename P::Seg, SegParamOut>::value) {
         using R = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::Refresh>;
         if (p.n_seeds == 1 && p.write_src != 0u)
             return launch<R>(one_seed_kernel<T, R, kAddToDst, OFF, P>, caches[2], p, ctas, job.stream);
@@ -820,9 +825,10 @@ cudaError_t launch_work(const Job& job, P& p) {
 
 // Packs segments, cut at multiples of kPieceElems, into launches whose pieces share the
 // high word of their block (checksum: window) indices.
-template <typename T, typename SEG>
+template <typename T, typename SEG, typename PAIR = SeedParam>
 cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size_t n_segs) {
-    using P = Launch<SEG, kParamBytes>;
+    using P = Launch<SEG, PAIR, kParamBytes>;
+    constexpr bool KEYED = std::is_same<PAIR, KeyedParam>::value;
     constexpr uint64_t E = Traits<T>::E, ES = sizeof(T);
     const uint64_t big_vec = 32ull * (job.work == kChecksum  ? Traits<T>::Sum::V
                                       : job.n_seeds == 1     ? Traits<T>::Pair::V  // = Refresh::V
@@ -831,6 +837,17 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
     uint64_t big_tiles = 0;
     for (size_t k = 0; k < n_segs; ++k) big_tiles += (segs[k].n + E * big_vec - 1) / (E * big_vec);
     const bool small = big_tiles < kSmallTiles;
+    // Pairs with their round keys are three times as long, so they are for tables that
+    // still fit one launch; the keys save 16 additions per pair and tile. Large shapes,
+    // 2^28 elements: update fp32 K = 16 4140 -> 4039 us, replay fp32 2744 -> 2622, bf16
+    // 2693 -> 2656; the bf16 update (4099 / 4108), the one-pair kernels (within 1%) and
+    // small tables (more parameters to copy) gain nothing.
+    constexpr bool MAY_KEY = std::is_same<SEG, SegParamOut>::value || std::is_same<T, float>::value;
+    if constexpr (MAY_KEY && !KEYED) {
+        if ((job.work == kUpdate || job.work == kGeneral) && job.n_seeds > 1 && !small &&
+            job.n_seeds * sizeof(KeyedParam) + (n_segs + 1) * sizeof(SEG) <= kParamBytes)
+            return enqueue_t<T, SEG, KeyedParam>(job, segs, dst, n_segs);
+    }
     bool split = false;
     if ((job.work == kUpdate || job.work == kGeneral) && job.n_seeds >= kSplitPairs && small) {
         uint64_t tiles = 0;
@@ -842,7 +859,7 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
     static thread_local P p;  // ~32 KB: keep it off the stack
     p.n_seeds = static_cast<uint32_t>(job.n_seeds);
     p.write_src = job.write_src ? 1u : 0u;
-    p.seg_at = static_cast<uint32_t>(job.n_seeds * sizeof(SeedParam));
+    p.seg_at = static_cast<uint32_t>(job.n_seeds * sizeof(PAIR));
     const size_t room = (P::kBytes - p.seg_at) / sizeof(SEG) - 1;  // and the sentinel
     SEG* table = reinterpret_cast<SEG*>(p.data + p.seg_at);
 
@@ -901,8 +918,8 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
         table[count].tile0 = static_cast<uint32_t>(tiles);
         p.n_segs = static_cast<uint32_t>(count);
         p.n_tiles = static_cast<uint32_t>(tiles);
-        SeedParam* sp = reinterpret_cast<SeedParam*>(p.data);
-        for (int k = 0; k < job.n_seeds; ++k) sp[k] = seed_param(job.seeds[k], hi, job.coef[k]);
+        PAIR* sp = reinterpret_cast<PAIR*>(p.data);
+        for (int k = 0; k < job.n_seeds; ++k) set_pair(sp[k], seed_param(job.seeds[k], hi, job.coef[k]));
         for (int k = 0; k < job.n_groups; ++k) sp[job.group_end[k] - 1].ends_group = 1u;
         if (job.work == kUpdate) sp[job.n_seeds - 1].ends_group = 1u;
         cudaError_t err;
@@ -920,11 +937,13 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
             }
         }
         const size_t used = p.seg_at + (count + 1) * sizeof(SEG);
-        if (split || (small && !off_grid)) {
+        if constexpr (KEYED) {
+            err = off_grid ? launch_work<T, false, true>(now, p) : launch_work<T, false, false>(now, p);
+        } else if (split || (small && !off_grid)) {
             if (used > kSmallParamBytes) {
                 err = split ? launch_split<T>(now, p) : launch_work<T, true, false>(now, p);
             } else {
-                Launch<SEG, kSmallParamBytes> q;
+                Launch<SEG, PAIR, kSmallParamBytes> q;
                 std::memcpy(&q, &p, offsetof(P, data) + used);
                 err = split ? launch_split<T>(now, q) : launch_work<T, true, false>(now, q);
             }

@@ -37,6 +37,7 @@
 // radius words and all angle words (|dz| <= 1e-6).
 #pragma once
 #include <cstdint>
+#include <type_traits>
 
 #include "jb_internal.h"
 
@@ -83,7 +84,8 @@ __device__ __forceinline__ BlockCtr block_ctr(uint32_t b_lo) {
 // block's product and constants of the pair; round 2 needs one product (the other one's
 // factor does not depend on the block's low word, so the host forms it, seed_param);
 // rounds 3 .. 10 in full: 17 wide multiplies.
-__device__ __forceinline__ uint4 philox_block(const SeedParam& s, const BlockCtr& c) {
+template <typename S>
+__device__ __forceinline__ uint4 philox_block(const S& s, const BlockCtr& c) {
     const uint64_t p1 = static_cast<uint64_t>(kPhiloxM1) * (c.p_hi ^ s.c2);
     uint32_t x0 = static_cast<uint32_t>(p1 >> 32) ^ s.c0;
     uint32_t x1 = static_cast<uint32_t>(p1);
@@ -92,6 +94,10 @@ __device__ __forceinline__ uint4 philox_block(const SeedParam& s, const BlockCtr
     uint32_t k0 = s.k0, k1 = s.k1;
 #pragma unroll
     for (int r = 2; r < 10; ++r) {
+        if constexpr (std::is_same<S, KeyedParam>::value) {
+            k0 = s.key[2 * (r - 2)];
+            k1 = s.key[2 * (r - 2) + 1];
+        }
         philox_round(x0, x1, x2, x3, k0, k1);
         k0 += kPhiloxW0;
         k1 += kPhiloxW1;

@@ -49,6 +49,8 @@ def operations(jb):
             "update K=1": lambda t: jb.jb_apply_updates(t, *pairs(1), LR, DENOM, QS),
             "update K=2": lambda t: jb.jb_apply_updates(t, *pairs(2), LR, DENOM, QS),
             "update K=5": lambda t: jb.jb_apply_updates(t, *pairs(5), LR, DENOM, QS),
+            # too many pairs for their round keys to travel with them
+            "update K=400": lambda t: jb.jb_apply_updates(t, *pairs(400), LR / 20, DENOM, QS),
             "from K=1": lambda t: into(t, 1), "from K=4": lambda t: into(t, 4), "replay": replay}
 
 
