@@ -223,8 +223,9 @@ __global__ void __launch_bounds__(kThreadsQ4) q4_perturb_kernel(const __grid_con
                 if constexpr (!ONE_HI) {
                     const uint64_t at = ((static_cast<uint64_t>(g.blk_hi) << 32) | g.blk0) + (i0 >> 2) + b;
                     sc = seed_param(p.seed, static_cast<uint32_t>(at >> 32), p.eps);
+                    return philox_block(sc, blk + b);
                 }
-                return philox_block(sc, blk + b);
+                return philox_block(sc, block_after(block_ctr(blk + (b & ~1)), b & 1));
             };
             uint4 wcur = words(0);
 #pragma unroll

@@ -80,6 +80,17 @@ __device__ __forceinline__ BlockCtr block_ctr(uint32_t b_lo) {
     return c;
 }
 
+// The same for the block that lies `delta` (a constant) further: an addition of 64 bits
+// instead of a multiplication. (Past the last block of the low word the result is not
+// that of the wrapped index; no element lies there.)
+__device__ __forceinline__ BlockCtr block_after(const BlockCtr& c, uint32_t delta) {
+    const uint64_t p = ((static_cast<uint64_t>(c.p_hi) << 32) | c.p_lo) + static_cast<uint64_t>(kPhiloxM0) * delta;
+    BlockCtr r;
+    r.p_hi = static_cast<uint32_t>(p >> 32);
+    r.p_lo = static_cast<uint32_t>(p);
+    return r;
+}
+
 // Four words of Philox4x32-10 for block c under the pair's constants. Round 1 is the
 // block's product and constants of the pair; round 2 needs one product (the other one's
 // factor does not depend on the block's low word, so the host forms it, seed_param);
