@@ -88,6 +88,21 @@ def aggregate_ranks(ms_local: float, units_local: float, dist=None, device=None)
     return float(mx[0].item()), float(t[1].item())
 
 
+def launches(table, pairs: int) -> int:
+    """Kernels of one in-place call: as many tensors as the 32 KB of parameters hold beside
+    the pairs, and no more than one high word of the Philox block index (2^34 elements)."""
+    room = (32704 - 32 * pairs) // 32 - 1
+    count, held, high = 0, 0, None
+    for numel, first in zip([t.numel() for t in table.tensors], table.flat_offsets):
+        at, end = first, first + numel
+        while at < end:
+            if held == room or at >> 34 != high:
+                count, held, high = count + 1, 0, at >> 34
+            held += 1
+            at = min(end, (at // (1 << 33) + 1) << 33)
+    return count
+
+
 def dist_env():
     return (int(os.environ.get("RANK", 0)), int(os.environ.get("LOCAL_RANK", 0)),
             int(os.environ.get("WORLD_SIZE", 1)))
@@ -264,7 +279,7 @@ def main():
     codes = [synthetic.byte_codes(K, 900, t) for t in range(n_total)]
     ghat = synthetic.rng(903).standard_normal(n_total) * 100.0
     stream = torch.cuda.current_stream()
-    launches_per_step = 3 * (-(-table.n_segments // 1000)) + (-(-table.n_segments // 700))
+    launches_per_step = 3 * launches(table, 1) + launches(table, K)
 
     ev = {}
 
@@ -331,7 +346,7 @@ def main():
     roofline = roof.report(K, upd_ms)
     roofline.update({
         "bound": "alu", "traffic": load_traffic(a),
-        "kernel": "seeded_kernel<bf16, update>" if a.dtype == "bf16" else "seeded_kernel<f32, update>",
+        "kernel": "seeded_kernel<bf16>" if a.dtype == "bf16" else "seeded_kernel<f32>",
         "perturb_ms": statistics.mean(pert_ms), "perturb_ms_best": min(pert_ms),
         "perturb_ms_median": statistics.median(pert_ms),
         "timing": f"CUDA events per launch over the {a.steps} timed steps; frac uses the best launch"})

@@ -44,19 +44,20 @@ namespace {
 // The shape of a kernel: vectors per thread and warp tile, threads per CTA (one CTA per
 // SM: the threads set how many registers each may use) and unrolling of the seed loop.
 // What bounds these kernels is the reading of operands and the issue of the instruction
-// mix (about 156 cycles per scheduler for a block's 95 instructions, 85% of them with the
-// FMA pipe that multiplies integers busy), not latency or memory, so the shapes differ
-// by a few percent. Measured on 2^28 elements (us), with the one-CTA alternatives:
+// mix (the bf16 update: 92 instructions and 153 cycles per scheduler for a warp's block and
+// pair, 83% of them with the FMA pipe that multiplies integers busy), not latency or
+// memory, so the shapes differ by a few percent. Measured on 2^28 elements (us):
 //   update, K = 16   fp32 5 x 512: 4137 (4 x 512: 4188, 4 x 768: 4202, 6 x 512: 4217)
 //                    bf16 3 x 512: 4099 (2 x 512: 4267, 2 x 768: 4157, 2 x 640: 4176)
 //   replay, 10 pairs fp32 4 x 512: 2655 (4 x 768: 2777, 6 x 512: 2766)
 //                    bf16 2 x 512: 2696 (2 x 768: 2755, 3 x 512: 2782)
-//   checksum         fp32 6 x 512: 152.0 (8 x 512: 153.4, 4 x 512: 157), bf16 79.9 (81.1, 83.2);
-//                    1.3B bf16 359 either way: 7.3 TB/s
-//   one pair that writes source and destination, fp32 (memory alone: 474): 16 warps per SM
-//                    4 x 512: 481; more of them in flight cost bandwidth (4 x 1024: 525)
 //   one pair         fp32 4 x 1024: 319 (4 x 768: 328, 4 x 512: 329; HBM alone: 316)
-//                    bf16 4 x 1024: 289 (4 x 768: 293, 4 x 512: 302, 8 x 768: 284)
+//                    bf16 4 x 1024: 283 (6 x 768: 280, 8 x 768: 284 and up to 14% slower
+//                    at 8M to 32M elements; before the last change 289, 4 x 512: 302)
+//   one pair that writes source and destination, fp32 (memory alone: 474): 16 warps per SM
+//                    4 x 512: 482; more of them in flight cost bandwidth (4 x 1024: 525)
+//   checksum         fp32 6 x 512: 152 (8 x 512: 153, 4 x 512: 157), bf16 80 (81, 83);
+//                    1.3B bf16 359: 7.3 TB/s
 // Small tables take one vector per thread in every kernel, and their launch fewer
 // parameter bytes: a scheduler needs about one warp's worth of blocks to be busy, so what
 // counts is that all 608 have some. The line lies where the large shape gives most of its
@@ -79,7 +80,7 @@ struct Traits<float> {
     using Update = Shape<5, 512, 2>;
     using General = Shape<4, 512, 2>;
     using Pair = Shape<4, 1024, 1>;
-    using Refresh = Shape<4, 512, 1, 1>;
+    using Refresh = Shape<4, 512, 1, 1>;  // one pair that writes the source too
     using Sum = Shape<6, 512, 1>;
     using Small = Shape<1, 512, 2>;
 };
@@ -128,7 +129,8 @@ __device__ __forceinline__ void store_vec(uint64_t a, uint4 w) { __stcs(reinterp
 
 // A whole vector at an address that is a multiple of `align` = 8, 4 or 2 bytes only: two
 // or four accesses, or, on an odd multiple of 2, the five words that it lies in (the
-// caller sees to it that they belong to the segment), of which the two at the ends are
+// caller sees to it that they belong to the segment; the outer halves of the two at the
+// ends are other vectors' elements, read and dropped), of which the two at the ends are
 // written by halves. A tensor off the 16-byte grid of its flat offset takes these, in
 // kernels of their own (OFF; in the common ones the choice costs registers). One
 // perturbation of 2^28 elements, against element by element: bf16 295 us at 8 bytes, 307
@@ -228,12 +230,12 @@ enum Store { kInPlace, kToDst, kNowhere };
 // x[j] is vector 32 j + lane of the tile in storage form, blk the low word of the first
 // Philox block of x[0] (x[j] is at blk + 32 j B; stored nowhere: of the window, and B is
 // 1), and present (stored nowhere only) how many vectors the segment has from x[0] on. A
-// warp takes spans of p.span
-// consecutive tiles, strided by the number of warps in the grid; tiles that follow one
-// another go to different SMs, so that a few tiles occupy as many SMs. Which warp
-// handles a tile never changes a result: every element's value depends only on its own
-// stored value, its global index and the seeds. Vectors that are partial (the ends of a
-// segment) go element by element. OFF: segments may lie off the 16-byte grid.
+// warp takes spans of p.span consecutive tiles, strided by the number of warps in the
+// grid; spans that follow one another go to different SMs, so that a few tiles occupy as
+// many SMs. Which warp handles a tile never changes a result: every element's value
+// depends only on its own stored value, its global index and the seeds. Vectors that are
+// partial (the ends of a segment) go element by element. OFF: segments may lie off the
+// 16-byte grid.
 template <typename T, typename S, Store TO, bool OFF, typename P, typename Op>
 __device__ __forceinline__ void visit_tiles(const P& p, bool also_src, Op&& op) {
     constexpr int E = Traits<T>::E, V = S::V;
@@ -809,6 +811,7 @@ cudaError_t launch_work(const Job& job, P& p) {
             return launch<U>(seeded_kernel<T, U, OFF, P>, caches[0], p, ctas, job.stream);
     } else if constexpr (std::is_same<typename P::Seg, SegParamOut>::value) {
         using R = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::Refresh>;
+        static_assert(R::V == S::V, "one table for both");
         if (p.n_seeds == 1 && p.write_src != 0u)
             return launch<R>(one_seed_kernel<T, R, kAddToDst, OFF, P>, caches[2], p, ctas, job.stream);
         if (p.n_seeds == 1)
