@@ -10,9 +10,9 @@ are measured by evaluating the fp32 Horner schemes exactly as the kernel does
 (each fused multiply-add rounded once to fp32) on a dense grid.
 
 Fitted functions (the kernel's variables):
-  P(w):  -2 ln f = 4 atanh(y) = sigma + y (sigma + w P(w)), sigma = 2(1 - f),
-         y = (1 - f) / (1 + f), w = y^2 in [0, 1/9] (f in [1/2, 1)); degree 2 would
-         leave a relative error of 2.0e-7
+  R(w):  ln(1 + t) = -q (1 + w R(w)) / 4 ... written through q = -4 s,
+         s = t / (2 + t), w = q^2, so that -2 ln(1 + t) = q + q w R(w);
+         w in [0, 16 s_max^2], s in [-1/7, 1/5] (t in [-1/4, 1/2)).
   S(y):  sin(pi x / 4) = x (pi/4 + y S(y)), y = x^2, x in [-1, 1];
          pi/4 is applied as hi + lo so that the leading term rounds once
   C(y):  cos(pi x / 4) = 1 + y C(y),  x in [-1, 1], C of degree 3 (degree 8 in x;
@@ -98,15 +98,19 @@ def hexf(x: float) -> str:
 
 
 def main():
-    # --- log: -2 ln f = sigma + y (sigma + w P(w)), w = y^2 ------------------------
-    def P_true(w):
+    # --- log: -2 ln(1 + t) = q + q w R(w), q = -4 t / (2 + t), w = q^2 -------------
+    smax = mp.mpf(1) / 5
+    wmax = 16 * smax ** 2
+    # with s^2 = w / 16:  -2 ln(1+t) = -4 atanh(s) = q (1 + s^2/3 + s^4/5 + ...)
+    #                     = q + q w R(w), R(w) = (atanh(s)/s - 1) / w
+    def R_true(w):
         if w == 0:
-            return mp.mpf(4) / 3
-        y = mp.sqrt(w)
-        return 4 * (mp.atanh(y) / y - 1) / w
-    # weight: error of y w P relative to 4 y
-    Pc = fit_rounded(P_true, [lambda w, k=k: w ** k for k in range(4)], 0, mp.mpf(1) / 9,
-                     lambda w: (w + mp.mpf("1e-30")) / 4)
+            return mp.mpf(1) / 48
+        s = mp.sqrt(w) / 4
+        return (mp.atanh(s) / s - 1) / w
+    basis = [lambda w, k=k: w ** k for k in range(3)]
+    # weight: error of q w R relative to q, i.e. w * (R - P)
+    Rc = fit_rounded(R_true, basis, 0, wmax, lambda w: w + mp.mpf("1e-30"))
     # --- sin(pi x / 4) = x S(x^2), x in [0, 1] ----------------------------------------
     def S_true(y):
         if y == 0:
@@ -143,18 +147,17 @@ def main():
     xs = x.astype(np.float64)
     es = np.max(np.abs(S[1:] - np.sin(np.pi * xs[1:] / 4)) / np.sin(np.pi * xs[1:] / 4))
     ec = np.max(np.abs(C - np.cos(np.pi * xs / 4)) / np.cos(np.pi * xs / 4))
-    f = np.linspace(0.5, 1, 300001)[:-1].astype(np.float32)
-    sg = fp32_fma(f, np.float32(-2), np.float32(2))
-    d = fp32_fma(f, np.float32(2), np.float32(2)).astype(np.float64)
-    yl = (sg.astype(np.float64) / d).astype(np.float32)
-    w = (yl.astype(np.float64) ** 2).astype(np.float32)
-    lf = fp32_fma(yl, fp32_fma(w, horner(Pc, w), sg), sg)
-    ref = -2 * np.log(f.astype(np.float64))
-    el = np.max(np.abs(lf - ref) / ref)
-    print("// P (log):", ", ".join(hexf(c) for c in Pc), f"   max rel err {el:.3e}")
+    t = np.linspace(-0.25, 0.5, 300001)[:-1].astype(np.float32)
+    q = (-4 * t.astype(np.float64) / (2 + t.astype(np.float64))).astype(np.float32)
+    w = (q.astype(np.float64) ** 2).astype(np.float32)
+    Lp = fp32_fma(q, (w.astype(np.float64) * horner(Rc, w)).astype(np.float32), q)  # degree 2
+    ref = -2 * np.log1p(t.astype(np.float64))
+    nz = ref != 0
+    el = np.max(np.abs(Lp[nz] - ref[nz]) / np.abs(ref[nz]))
+    print("// R (log):", ", ".join(hexf(c) for c in Rc), f"   max rel err {el:.3e} (q exact)")
     print("// S (sin):", ", ".join(hexf(c) for c in Sc), f"   max rel err {es:.3e}")
     print("// C (cos):", ", ".join(hexf(c) for c in Cc), f"   max rel err {ec:.3e}")
-    for name, cs in (("kLogP", Pc), ("kSinS", Sc), ("kCosC", Cc)):
+    for name, cs in (("kLogR", Rc), ("kSinS", Sc), ("kCosC", Cc)):
         print(f"constexpr float {name}[{len(cs)}] = {{" + ", ".join(hexf(c) + "f" for c in cs) + "};")
 
 

@@ -11,14 +11,11 @@
 // Nothing here is written to memory on the hot path.
 //
 // Arithmetic of the transform (fp32, every rounding explicit):
-//   radius  u_a = 2^e f exactly, f in [1/2, 1), with sigma = 2(1 - f) exact and
-//           y = sigma / (2(1 + f)) (one rcp.approx):
-//           -2 ln f = 4 atanh(y) = sigma + y (sigma + w P(w)), w = y^2, P a degree-3
-//           minimax polynomial. The leading term is exact, so the error of the
-//           reciprocal enters only through the second term (at most 0.28 of the sum);
-//           u_a near 1 has e = 0 and keeps its relative accuracy.
-//           L = -2 ln f - e (2 ln 2) (2 ln 2 in fp32 is within 2.8e-9, so one product
-//           is enough); r = sqrt.approx(L) (relative error below 1.1e-7 over every L).
+//   radius  u_a = 2^e f exactly, f in [3/4, 3/2), t = f - 1 exact; with
+//           q = 4t / (2 + t) (one rcp.approx), 2 ln f = q + q w R(w), w = q^2, R a
+//           degree-2 minimax polynomial; 2 ln u_a = e (2 ln 2) + 2 ln f with 2 ln 2
+//           split hi + lo (Cody & Waite 1980) so that e (2 ln 2)_hi is exact;
+//           r = sqrt.approx(-2 ln u_a) (relative error below 1.1e-7 over all of them).
 //   angle   with t = x_b + 2^29, the angle is q pi/2 + (pi/4) x, q = t >> 30, x in
 //           (-1, 1) exact from the 22 bits below; sin and cos of (pi/4) x by minimax
 //           polynomials of degree 7 and 8 (relative error < 0.6 ulp for the sine, also
@@ -26,12 +23,16 @@
 //           (and negates the sine), q >= 2 flips both: that sign goes to the radius.
 // Integers become floats by placing their bits under a constant exponent (one shift,
 // at most one mask, and a subtraction that the packed arithmetic does for two): an
-// integer-to-float conversion costs more issue slots than those. Against f in
-// [3/4, 3/2) with integer conversions, and an octant reflection with both signs applied
-// to the results, one pass over 1.3B bf16 elements went from 1653 to 1524 us (one pair)
-// and a K = 16 update of 125M fp32 elements from 2239 to 2123 us; it is also more
-// accurate: rms |dz| 4.75e-8 -> 4.69e-8, largest over 1.3e8 draws 8.0e-7 -> 7.5e-7,
-// joint worst case 8.7e-7 -> 8.2e-7.
+// integer-to-float conversion costs more issue slots than those. e and the scale of f come
+// from the exponent of (4/3) u_a, one packed product for two radii; an integer addition for
+// each costs 1.2 to 1.7 % more (one pair over 1.3B bf16 elements 1401 against 1380 us, a
+// K = 16 update of 125M fp32 elements 1966 against 1932). The signs of the half turn go to
+// the radius. Every rounding is that of integer conversions, an octant reflection and
+// signs applied to the results, so the bits of z are too; in these kernels that form takes
+// 6 to 13 % more (1509 against 1424 us for the one-pair update of 1.3B bf16 elements, 2180
+// against 1934 for the fp32 update). A leading term 2(1 - f) with f in [1/2, 1) would be up
+// to 2 % faster still and a little more accurate, but gives other bits: a replay rounds to
+// bf16 many times, and a late joiner must end with the weights of those that trained on.
 // Coefficients: fit_poly.py (Remez exchange). The transform is checked
 // against a double-precision evaluation of the same definition over all
 // radius words and all angle words (|dz| <= 1e-6).
@@ -44,14 +45,15 @@
 namespace jb {
 
 // Polynomials (fit_poly.py).
-constexpr float kLogP0 = 0x1.5555p+0f, kLogP1 = 0x1.99d29ep-1f, kLogP2 = 0x1.1eb3a2p-1f,
-                kLogP3 = 0x1.1f0578p-1f;
+constexpr float kLogR0 = 0x1.5555b4p-6f, kLogR1 = 0x1.992aaap-11f, kLogR2 = 0x1.36ec6ap-15f;
 constexpr float kSinHi = 0x1.921fb6p-1f;   // pi/4 = hi + lo
 constexpr float kSinLo = -0x1.777a5cp-26f;
 constexpr float kSinS0 = -0x1.4abbbep-4f, kSinS1 = 0x1.465facp-9f, kSinS2 = -0x1.2db5cep-15f;
 constexpr float kCosC0 = -0x1.3bd3ccp-2f, kCosC1 = 0x1.03c1b0p-6f, kCosC2 = -0x1.55b2b6p-12f,
                 kCosC3 = 0x1.d4f7eep-19f;
-constexpr float kTwoLn2 = 0x1.62e430p+0f;
+constexpr float kTwoLn2Hi = 0x1.62e4p+0f;       // 2 ln 2 to 16 bits
+constexpr float kTwoLn2Lo = 0x1.7f7d1cp-19f;   // 2 ln 2 - kTwoLn2Hi
+
 
 // One Philox round on (x0, x1, x2, x3) with round key (k0, k1).
 __device__ __forceinline__ void philox_round(uint32_t& x0, uint32_t& x1, uint32_t& x2,
@@ -155,32 +157,29 @@ __device__ __forceinline__ float shift_under(uint32_t hi, uint32_t lo, int n) {
     return __uint_as_float(__funnelshift_r(lo, hi, n));
 }
 
-// (bits & keep) | set in one instruction
-__device__ __forceinline__ float masked(uint32_t bits, uint32_t keep, uint32_t set) {
-    uint32_t r;
-    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(r) : "r"(bits), "r"(keep), "r"(set));
-    return __uint_as_float(r);
-}
-
 __device__ __forceinline__ Polar2 polar2(uint4 w) {
     // ---- radius ----
-    // 1 + (x_a >> 9) 2^-23, less 1 - 2^-24: u_a, exact
-    const float2 u = add2(make_float2(shift_under(0x7Fu, w.x, 9), shift_under(0x7Fu, w.z, 9)),
-                          splat(-0x1.fffffep-1f));
-    const uint32_t uA = __float_as_uint(u.x), uB = __float_as_uint(u.y);
-    const float2 f = make_float2(masked(uA, 0x7FFFFFu, 0x3F000000u), masked(uB, 0x7FFFFFu, 0x3F000000u));
-    // 2^23 + biased exponent, less 2^23 + 126: e, exact
-    const float2 e = add2(make_float2(shift_under(0x4B000000u >> 9, uA, 23),
-                                      shift_under(0x4B000000u >> 9, uB, 23)), splat(-8388734.0f));
-    const float2 sg = fma2(f, splat(-2.0f), splat(2.0f));             // 2(1 - f), exact
-    const float2 d = fma2(f, splat(2.0f), splat(2.0f));
-    const float2 y = mul2(sg, make_float2(rcp_approx(d.x), rcp_approx(d.y)));  // (1 - f) / (1 + f)
-    const float2 ww = mul2(y, y);
-    float2 p = fma2(ww, splat(kLogP3), splat(kLogP2));
-    p = fma2(ww, p, splat(kLogP1));
-    p = fma2(ww, p, splat(kLogP0));
-    const float2 lf = fma2(y, fma2(ww, p, sg), sg);                   // -2 ln f
-    const float2 L = fma2(e, splat(-kTwoLn2), lf);                    // -2 ln u_a
+    // 1/2 + (x_a >> 9) 2^-24, less 1/2 - 2^-25: u_a / 2, exact
+    const float2 u = add2(make_float2(shift_under(0x7Eu, w.x, 9), shift_under(0x7Eu, w.z, 9)),
+                          splat(-0x1.fffffep-2f));
+    // times 4/3 (and 2): the exponent steps where f passes 3/4; fp32's 8/3 does it at the
+    // right word for all 2^23 of them
+    const float2 v = mul2(u, splat(0x1.555556p+1f));
+    const uint32_t hA = __float_as_uint(v.x), hB = __float_as_uint(v.y);
+    // 2^23 + biased exponent, less 2^23 + 127: e, exact
+    const float2 e = add2(make_float2(shift_under(0x4B000000u >> 9, hA, 23),
+                                      shift_under(0x4B000000u >> 9, hB, 23)), splat(-8388735.0f));
+    // the exponent's complement is that of 2^(1 - e): t = f - 1, exact
+    const float2 t = fma2(u, make_float2(__uint_as_float(~hA & 0x7F800000u),
+                                         __uint_as_float(~hB & 0x7F800000u)), splat(-1.0f));
+    const float2 d = fma2(t, splat(0.25f), splat(0.5f));                // (2 + t) / 4
+    const float2 q = mul2(t, make_float2(rcp_approx(d.x), rcp_approx(d.y)));  // 4t / (2 + t)
+    const float2 ww = mul2(q, q);
+    float2 p = fma2(ww, splat(kLogR2), splat(kLogR1));
+    p = fma2(ww, p, splat(kLogR0));
+    const float2 lp = fma2(q, mul2(ww, p), q);                          // 2 ln f
+    // e (2 ln 2)_hi is exact, so L is the sum of it and the rest rounded once
+    const float2 L = fma2(e, splat(kTwoLn2Hi), fma2(e, splat(kTwoLn2Lo), lp));  // 2 ln u_a
 
     // ---- angle ----
     const uint32_t tA = w.y + 0x20000000u, tB = w.w + 0x20000000u;
@@ -201,8 +200,8 @@ __device__ __forceinline__ Polar2 polar2(uint4 w) {
     const bool swA = (tA & 0x40000000u) != 0u, swB = (tB & 0x40000000u) != 0u;
     Polar2 o;
     o.rr = make_float2(
-        __uint_as_float(__float_as_uint(sqrt_approx(L.x)) ^ (tA & 0x80000000u)),
-        __uint_as_float(__float_as_uint(sqrt_approx(L.y)) ^ (tB & 0x80000000u)));
+        __uint_as_float(__float_as_uint(sqrt_approx(-L.x)) ^ (tA & 0x80000000u)),
+        __uint_as_float(__float_as_uint(sqrt_approx(-L.y)) ^ (tB & 0x80000000u)));
     o.cm = make_float2(swA ? -S.x : C.x, swB ? -S.y : C.y);
     o.sm = make_float2(swA ? C.x : S.x, swB ? C.y : S.y);
     return o;
