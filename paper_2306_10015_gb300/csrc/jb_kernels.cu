@@ -44,16 +44,17 @@ namespace {
 // The shape of a kernel: vectors per thread and warp tile, threads per CTA (one CTA per
 // SM: the threads set how many registers each may use) and unrolling of the seed loop.
 // What bounds these kernels is the reading of operands and the issue of the instruction
-// mix (the bf16 update: 92 instructions and 153 cycles per scheduler for a warp's block and
-// pair, 83% of them with the FMA pipe that multiplies integers busy), not latency or
+// mix (the bf16 update: 92 instructions and 155 cycles per scheduler for a warp's block and
+// pair, 82% of them with the FMA pipe that multiplies integers busy), not latency or
 // memory, so the shapes differ by a few percent. Measured on 2^28 elements (us):
-//   update, K = 16   fp32 5 x 512: 4137 (4 x 512: 4188, 4 x 768: 4202, 6 x 512: 4217)
-//                    bf16 3 x 512: 4099 (2 x 512: 4267, 2 x 768: 4157, 2 x 640: 4176)
-//   replay, 10 pairs fp32 4 x 512: 2655 (4 x 768: 2777, 6 x 512: 2766)
-//                    bf16 2 x 512: 2696 (2 x 768: 2755, 3 x 512: 2782)
-//   one pair         fp32 4 x 1024: 319 (4 x 768: 328, 4 x 512: 329; HBM alone: 316)
-//                    bf16 4 x 1024: 283 (6 x 768: 280, 8 x 768: 284 and up to 14% slower
-//                    at 8M to 32M elements; before the last change 289, 4 x 512: 302)
+//   update, K = 16   fp32 5 x 512: 4111 (4 x 512: 4147, 4 x 768: 4171, 6 x 512: 4156)
+//                    bf16 3 x 512: 4163 (2 x 512: 4332, 2 x 768: 4171, 2 x 640: 4156)
+//   replay, 10 pairs fp32 4 x 512: 2663 (4 x 768: 2871, 6 x 512: 2812)
+//                    bf16 2 x 512: 2667 (2 x 768: 2794, 3 x 512: 2817)
+//   one pair         fp32 4 x 1024: 318 (4 x 768: 338, 4 x 512: 329; HBM alone: 316)
+//                    bf16 4 x 1024: 282 and 291 (perturbation, update; 6 x 768: 286 and 290,
+//                    8 x 768: 284 and 285, but up to 14% slower at 8M to 32M elements;
+//                    4 x 512: 306 and 303)
 //   one pair that writes source and destination, fp32 (memory alone: 474): 16 warps per SM
 //                    4 x 512: 482; more of them in flight cost bandwidth (4 x 1024: 525)
 //   checksum         fp32 6 x 512: 152 (8 x 512: 153, 4 x 512: 157), bf16 80 (81, 83);
@@ -61,8 +62,9 @@ namespace {
 // Small tables take one vector per thread in every kernel, and their launch fewer
 // parameter bytes: a scheduler needs about one warp's worth of blocks to be busy, so what
 // counts is that all 608 have some. The line lies where the large shape gives most of its
-// 16 warps per SM a tile (K = 32 update, us, one vector / large shape; fp32 512K elements
-// 27 / 29, 1M 43 / 40, 2M 84 / 77; bf16 512K 25 / 33, 1M 43 / 47, 1.5M 62 / 59, 3M 111 / 103).
+// 16 warps per SM a tile (K = 32 update, us, one vector / large shape: fp32 512K elements
+// 27 / 29, 1M 43 / 39, 2M 84 / 76; bf16 256K 23 / 25, 512K 25 / 35, 1M 43 / 47, 1.5M 62 / 61,
+// 3M 111 / 104).
 template <int V_, int THREADS_, int UNROLL_, int CTAS_ = 0>
 struct Shape {
     static constexpr int V = V_, THREADS = THREADS_, UNROLL = UNROLL_;
@@ -133,8 +135,8 @@ __device__ __forceinline__ void store_vec(uint64_t a, uint4 w) { __stcs(reinterp
 // ends are other vectors' elements, read and dropped), of which the two at the ends are
 // written by halves. A tensor off the 16-byte grid of its flat offset takes these, in
 // kernels of their own (OFF; in the common ones the choice costs registers). One
-// perturbation of 2^28 elements, against element by element: bf16 295 us at 8 bytes, 307
-// at 4, 415 at 2 (541 to 615 before; 289 on the grid), fp32 343 and 360 (427; 318).
+// perturbation of 2^28 elements, against element by element: bf16 295 us at 8 bytes, 306
+// at 4, 411 at 2 (541 to 615 before; 281 on the grid), fp32 350 and 368 (427; 317).
 __device__ __forceinline__ uint4 load_off_grid(uint64_t a, uint32_t align) {
     uint4 w;
     if (align == 8u) {
@@ -481,10 +483,10 @@ __global__ void __launch_bounds__(S::THREADS) general_update_kernel(const __grid
 // update_tile, so the results are the same bit for bit. One warp alone needs about 350
 // cycles per pair for a tile (the latency of the generator and the transform; 580 where a
 // thread has the two blocks of a bf16 vector); shared out, an SM needs about 40. K = 400
-// update, us, before and with the split: fp32 1K to 19K elements 68 and 27, 65K 84 and 53,
-// 78K 84 and 93; bf16 1K 115 and 31, 65K 115 and 53, 160K 148 and 117, 262K 148 and 175.
-// So it ends at one tile per scheduler (608) in fp32 and at two in bf16. It is not slower
-// for two pairs either (4.9 -> 3.3 us for 1K bf16 elements).
+// update, us, without and with the split: fp32 1K to 19K elements 70 and 29, 65K 85 and 62,
+// 78K 85 and 96; bf16 1K 117 and 31, 65K 119 and 62, 131K 150 and 112, 160K 150 and 156,
+// 262K 150 and 222. So it ends at one tile per scheduler (608) in fp32 and at two in bf16.
+// It is not slower for two pairs either (5.7 and 5.8 us for 1K elements, bound by the call).
 constexpr int kSplitThreads = 512;
 constexpr int kSplitWarps = kSplitThreads / 32;
 constexpr int kSplitPairs = 2;
@@ -843,11 +845,11 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
     for (size_t k = 0; k < n_segs; ++k) big_tiles += (segs[k].n + E * big_vec - 1) / (E * big_vec);
     const bool small = big_tiles < kSmallTiles;
     // Pairs with their round keys are three times as long, so they are for tables that
-    // still fit one launch; the keys save 16 additions per pair and tile. Large shapes,
-    // 2^28 elements: update fp32 K = 16 4140 -> 4039 us, replay fp32 2744 -> 2622, bf16
-    // 2693 -> 2656; the bf16 update (4099 / 4108), the one-pair kernels (within 1%) and
-    // small tables (more parameters to copy) gain nothing.
-    constexpr bool MAY_KEY = std::is_same<SEG, SegParamOut>::value || std::is_same<T, float>::value;
+    // still fit one launch; the keys save 16 additions per pair and tile. fp32, 2^28
+    // elements: update K = 16 4128 -> 4111 us, replay 2713 -> 2663. The bf16 replay is
+    // faster without keys (2667 / 2694); the bf16 update, the one-pair kernels and small
+    // tables (more parameters to copy) gain nothing.
+    constexpr bool MAY_KEY = std::is_same<T, float>::value;
     if constexpr (MAY_KEY && !KEYED) {
         if ((job.work == kUpdate || job.work == kGeneral) && job.n_seeds > 1 && !small &&
             job.n_seeds * sizeof(KeyedParam) + (n_segs + 1) * sizeof(SEG) <= kParamBytes)

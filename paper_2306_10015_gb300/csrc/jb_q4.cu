@@ -133,7 +133,7 @@ __device__ __forceinline__ void dequant_block(const float2* pair, const uint32_t
     lo = pair_at<B % 2, true>(pair, cw[B / 2]);
 }
 
-constexpr int kThreadsQ4 = 768;
+constexpr int kThreadsQ4 = 1024;
 
 template <typename P>
 __device__ __forceinline__ const SegParamQ4& q4_seg(const P& p, uint32_t s) {
@@ -142,10 +142,11 @@ __device__ __forceinline__ const SegParamQ4& q4_seg(const P& p, uint32_t s) {
 
 // A warp tile is 1024 consecutive elements of one tensor, 32 per lane; tiles and spans as
 // in the update's kernels. Bound, like those, by operand reads and the instruction mix
-// (139 instructions and 229 cycles per scheduler and four elements of a warp; FMA pipe 73%
-// busy, shared-memory reads 39%). Six warps per scheduler at 80 registers: 2^28 elements
-// in 357 us (640 threads 363, 1024 threads 360, 512 threads 371); 397 before, with lanes
-// numbered across tensors, codes shifted into place and bank conflicts on the buckets.
+// (147 instructions and 237 cycles per scheduler and four elements of a warp at 768
+// threads; FMA pipe 72% busy, shared-memory reads 36%). Eight warps per scheduler at 64
+// registers: 2^28 elements in 358 us (768 threads 364, 640 threads 365, 512 threads 386);
+// 397 before, with lanes numbered across tensors, codes shifted into place and bank
+// conflicts on the buckets.
 // ONE_HI: the pair's constants hold for every block of the launch; otherwise they are
 // formed for the high word of each block's own index.
 template <bool ONE_HI, typename P>
