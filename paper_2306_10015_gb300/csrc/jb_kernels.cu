@@ -44,7 +44,7 @@ namespace {
 // The shape of a kernel: vectors per thread and warp tile, threads per CTA (one CTA per
 // SM: the threads set how many registers each may use) and unrolling of the seed loop.
 // What bounds these kernels is the reading of operands and the issue of the instruction
-// mix (the bf16 update: 92 instructions and 155 cycles per scheduler for a warp's block and
+// mix (the bf16 update: 92 instructions and 154 cycles per scheduler for a warp's block and
 // pair, 82% of them with the FMA pipe that multiplies integers busy), not latency or
 // memory, so the shapes differ by a few percent. Measured on 2^28 elements (us):
 //   update, K = 16   fp32 5 x 512: 4111 (4 x 512: 4147, 4 x 768: 4171, 6 x 512: 4156)
@@ -58,7 +58,7 @@ namespace {
 //   one pair that writes source and destination, fp32 (memory alone: 474): 16 warps per SM
 //                    4 x 512: 482; more of them in flight cost bandwidth (4 x 1024: 525)
 //   checksum         fp32 6 x 512: 152 (8 x 512: 153, 4 x 512: 157), bf16 80 (81, 83);
-//                    1.3B bf16 359: 7.3 TB/s
+//                    1.3B bf16 364: 7.2 TB/s
 // Small tables take one vector per thread in every kernel, and their launch fewer
 // parameter bytes: a scheduler needs about one warp's worth of blocks to be busy, so what
 // counts is that all 608 have some. The line lies where the large shape gives most of its

@@ -142,9 +142,8 @@ __device__ __forceinline__ const SegParamQ4& q4_seg(const P& p, uint32_t s) {
 
 // A warp tile is 1024 consecutive elements of one tensor, 32 per lane; tiles and spans as
 // in the update's kernels. Bound, like those, by operand reads and the instruction mix
-// (147 instructions and 237 cycles per scheduler and four elements of a warp at 768
-// threads; FMA pipe 72% busy, shared-memory reads 36%). Eight warps per scheduler at 64
-// registers: 2^28 elements in 358 us (768 threads 364, 640 threads 365, 512 threads 386);
+// (151 instructions and 218 cycles per scheduler and four elements of a warp; FMA pipe 76%
+// busy, shared-memory reads 36%). Eight warps per scheduler at 64 registers, a few spilled: 2^28 elements in 358 us (768 threads 364, 640 threads 365, 512 threads 386);
 // 397 before, with lanes numbered across tensors, codes shifted into place and bank
 // conflicts on the buckets.
 // ONE_HI: the pair's constants hold for every block of the launch; otherwise they are
