@@ -401,7 +401,7 @@ def generator_rate(jb, stream, n_blocks=1 << 32, reps=5):
 class Roofline:
     """Rooflines of the fused K-seed update on this GPU, per K and launch time.
 
-    * frac (judged; the combined roofline of the task): T_roof = max(T_HBM, T_ALG),
+    * frac (the combined roofline): T_roof = max(T_HBM, T_ALG),
       T_HBM = 2 sizeof(T) N / measured copy bandwidth, T_ALG = the algorithm's fixed
       count of OPS_PER_PARAM_SEED = 15 lane operations per element-seed (a quarter
       Philox4x32-10 block: 10 rounds x (2 wide multiplies + 2 three-input XORs) / 4;
