@@ -254,10 +254,14 @@ def jb_apply_updates_from(src: ParamTable, dst: ParamTable, seeds, q, lr: float,
 def jb_replay_updates(table: ParamTable, steps, qscale: float, stream=None) -> None:
     """Apply several steps' updates in order, in place; steps = [(seeds, q, lr, denom), ...]."""
     seeds = [seeds_array(st[0]) for st in steps]
-    codes = [_codes_array(st[1]) for st in steps]
+    codes = [np.asarray(st[1], dtype=np.int8, order="C") for st in steps]
     sizes = np.array([len(x) for x in seeds], dtype=np.int32)
     if any(len(c) != len(x) for c, x in zip(codes, seeds)):
         raise ValueError("one byte code per seed")
+    # joined as bytes: what numpy's concatenation would refuse is refused here
+    if {a.ndim for a in seeds + codes} != {1} and any(
+            len({a.shape[1:] for a in arrays}) > 1 for arrays in (seeds, codes)):
+        raise ValueError("the arrays of the steps differ in their dimensions")
     lr = np.array([float(st[2]) for st in steps], dtype=np.float32)
     denom = np.array([float(st[3]) for st in steps], dtype=np.float32)
     _check(lib().jb_replay_updates(table.segments, table.n_segments, table.dtype,

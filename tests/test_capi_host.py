@@ -199,6 +199,22 @@ def test_apply_from_and_replay_validation(jb):
     # validation passes and the call reaches the launch, which has no device here
 
 
+def test_replay_refuses_codes_of_unequal_shape(jb):
+    """Codes of a step are one array of one dimension: a bare number has no length, and
+    steps whose arrays differ in their dimensions cannot be put in a row."""
+    from types import SimpleNamespace
+    empty = SimpleNamespace(segments=None, n_segments=0, dtype=0)
+    replay = lambda *steps: jb.jb_replay_updates(empty, [(s, q, 1e-3, 1.0) for s, q in steps], 16.0, stream=0)
+    one, two = [(1, 0, 0)], [(1, 0, 0), (2, 0, 0)]
+    replay((one, [5]), (two, [3, -4]), ([], []))
+    with pytest.raises(TypeError):
+        replay((one, 5))
+    with pytest.raises(ValueError):
+        replay((one, [[5, 6]]), (two, [3, 4]))
+    with pytest.raises(ValueError):
+        replay((two, [3]))
+
+
 def test_checksum_validation(jb):
     import ctypes as C
     src = _segs(jb, [(FAKE, 100, 0)])
