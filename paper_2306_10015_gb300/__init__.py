@@ -120,9 +120,11 @@ def _check(rc: int) -> None:
 def _stream(stream) -> ctypes.c_void_p:
     if stream is None:
         import torch
-        if torch.cuda.is_initialized():
-            # the current stream's handle without a Stream object around it (0.1 us, not 3)
-            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        # the current stream's handle without a Stream object around it (0.1 us, not 3); the
+        # function is not part of torch's public interface, so it may be missing
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None and torch.cuda.is_initialized():
+            return ctypes.c_void_p(raw(torch.cuda.current_device()))
         return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     if isinstance(stream, int):
         return ctypes.c_void_p(stream)

@@ -144,6 +144,20 @@ def test_invalid_arguments(jb):
     assert _update(jb, ok, 1, many, [1] * K) == E["many"]
 
 
+@pytest.mark.parametrize("raw", [True, False])
+def test_default_stream_with_and_without_the_raw_handle(jb, monkeypatch, raw):
+    """The current stream is found on a torch that lacks the private function for its handle."""
+    import torch
+    from types import SimpleNamespace
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: SimpleNamespace(cuda_stream=0x1230))
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 0x4560 + device, raising=False)
+    if not raw:
+        monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream")
+    assert jb._stream(None).value == (0x4563 if raw else 0x1230)
+
+
 def test_python_table_rejects_cpu_tensors(jb):
     import torch
     with pytest.raises(ValueError):
