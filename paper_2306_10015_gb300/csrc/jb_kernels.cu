@@ -36,6 +36,7 @@
 #include <type_traits>
 
 #include "jb_internal.h"
+#include "jb_offgrid.h"
 #include "jb_rng.cuh"
 
 namespace jb {
@@ -129,49 +130,18 @@ __device__ __forceinline__ uint4 pack(const float2 (&x)[2][2]) {
 __device__ __forceinline__ uint4 load_vec(uint64_t a) { return __ldcs(reinterpret_cast<const uint4*>(a)); }
 __device__ __forceinline__ void store_vec(uint64_t a, uint4 w) { __stcs(reinterpret_cast<uint4*>(a), w); }
 
-// A whole vector at an address that is a multiple of `align` = 8, 4 or 2 bytes only: two
-// or four accesses, or, on an odd multiple of 2, the five words that it lies in (the
-// caller sees to it that they belong to the segment; the outer halves of the two at the
-// ends are other vectors' elements, read and dropped), of which the two at the ends are
-// written by halves. A tensor off the 16-byte grid of its flat offset takes these, in
-// kernels of their own (OFF; in the common ones the choice costs registers). One
+// Memory for the vectors off the 16-byte grid of their flat offset (jb_offgrid.h). They
+// take kernels of their own (OFF; in the common ones the choice costs registers). One
 // perturbation of 2^28 elements, against element by element: bf16 295 us at 8 bytes, 306
 // at 4, 411 at 2 (541 to 615 before; 281 on the grid), fp32 350 and 368 (427; 317).
-__device__ __forceinline__ uint4 load_off_grid(uint64_t a, uint32_t align) {
-    uint4 w;
-    if (align == 8u) {
-        const uint2 p = __ldcs(reinterpret_cast<const uint2*>(a)), q = __ldcs(reinterpret_cast<const uint2*>(a) + 1);
-        w = make_uint4(p.x, p.y, q.x, q.y);
-    } else if (align == 4u) {
-        const uint32_t* p = reinterpret_cast<const uint32_t*>(a);
-        w = make_uint4(__ldcs(p), __ldcs(p + 1), __ldcs(p + 2), __ldcs(p + 3));
-    } else {
-        const uint32_t* p = reinterpret_cast<const uint32_t*>(a - 2);
-        const uint32_t q[5] = {__ldcs(p), __ldcs(p + 1), __ldcs(p + 2), __ldcs(p + 3), __ldcs(p + 4)};
-        w = make_uint4(__funnelshift_r(q[0], q[1], 16), __funnelshift_r(q[1], q[2], 16),
-                       __funnelshift_r(q[2], q[3], 16), __funnelshift_r(q[3], q[4], 16));
-    }
-    return w;
-}
-__device__ __forceinline__ void store_off_grid(uint64_t a, uint32_t align, uint4 w) {
-    if (align == 8u) {
-        __stcs(reinterpret_cast<uint2*>(a), make_uint2(w.x, w.y));
-        __stcs(reinterpret_cast<uint2*>(a) + 1, make_uint2(w.z, w.w));
-    } else if (align == 4u) {
-        uint32_t* p = reinterpret_cast<uint32_t*>(a);
-        __stcs(p, w.x);
-        __stcs(p + 1, w.y);
-        __stcs(p + 2, w.z);
-        __stcs(p + 3, w.w);
-    } else {
-        *reinterpret_cast<uint16_t*>(a) = static_cast<uint16_t>(w.x);
-        uint32_t* p = reinterpret_cast<uint32_t*>(a + 2);
-        __stcs(p, __funnelshift_r(w.x, w.y, 16));
-        __stcs(p + 1, __funnelshift_r(w.y, w.z, 16));
-        __stcs(p + 2, __funnelshift_r(w.z, w.w, 16));
-        *reinterpret_cast<uint16_t*>(a + 14) = static_cast<uint16_t>(w.w >> 16);
-    }
-}
+struct Global {
+    __device__ uint2 load64(uint64_t a) const { return __ldcs(reinterpret_cast<const uint2*>(a)); }
+    __device__ uint32_t load32(uint64_t a) const { return __ldcs(reinterpret_cast<const uint32_t*>(a)); }
+    __device__ uint16_t load16(uint64_t a) const { return *reinterpret_cast<const uint16_t*>(a); }
+    __device__ void store64(uint64_t a, uint2 v) const { __stcs(reinterpret_cast<uint2*>(a), v); }
+    __device__ void store32(uint64_t a, uint32_t v) const { __stcs(reinterpret_cast<uint32_t*>(a), v); }
+    __device__ void store16(uint64_t a, uint16_t v) const { *reinterpret_cast<uint16_t*>(a) = v; }
+};
 
 // Elements [first, last) of the window at address a (the others read as zero bits).
 template <typename T>
@@ -270,7 +240,7 @@ __device__ __forceinline__ void visit_tiles(const P& p, bool also_src, Op&& op) 
                     for (int j = 0; j < V; ++j) x[j] = load_vec(src + 512ull * j);
                 } else if (fast) {
 #pragma unroll
-                    for (int j = 0; j < V; ++j) x[j] = load_off_grid(src + 512ull * j, load_align);
+                    for (int j = 0; j < V; ++j) x[j] = load_off_grid(Global(), src + 512ull * j, load_align);
                 } else {
 #pragma unroll
                     for (int j = 0; j < V; ++j) {
@@ -299,16 +269,16 @@ __device__ __forceinline__ void visit_tiles(const P& p, bool also_src, Op&& op) 
                         store_vec(out + 512ull * j, x[j]);
                         if (TO_DST && also_src) {
                             if (load_align == 16u) store_vec(src + 512ull * j, x[j]);
-                            else store_off_grid(src + 512ull * j, load_align, x[j]);
+                            else store_off_grid(Global(), src + 512ull * j, load_align, x[j]);
                         }
                     }
                 } else if (fast) {
 #pragma unroll
                     for (int j = 0; j < V; ++j) {
-                        store_off_grid(out + 512ull * j, store_align, x[j]);
+                        store_off_grid(Global(), out + 512ull * j, store_align, x[j]);
                         if (TO_DST && also_src) {
                             if (load_align == 16u) store_vec(src + 512ull * j, x[j]);
-                            else store_off_grid(src + 512ull * j, load_align, x[j]);
+                            else store_off_grid(Global(), src + 512ull * j, load_align, x[j]);
                         }
                     }
                 } else {
@@ -907,13 +877,7 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
             if (g.load != size || g.store != size) off_grid = true;
             g.lo = head != 0 ? 1 : 0;
             g.full = static_cast<uint32_t>(g.end / win);
-            if (split) {
-                if (g.load != size || g.store != size) g.full = 0;  // element by element
-            } else if (g.load == 2 || g.store == 2) {
-                // reads and writes reach two bytes past a vector on both sides
-                g.lo += 1;
-                g.full = g.full > 1 ? g.full - 1 : 0;
-            }
+            if (split && (g.load != size || g.store != size)) g.full = 0;  // element by element
             const uint64_t vecs = (g.end + win - 1) / win;
             tiles += (vecs + tile_vec - 1) / tile_vec;
             at += n;
