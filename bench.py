@@ -90,7 +90,8 @@ def aggregate_ranks(ms_local: float, units_local: float, dist=None, device=None)
 
 def launches(table, pairs: int) -> int:
     """Kernels of one in-place call: as many tensors as the 32 KB of parameters hold beside
-    the pairs, and no more than one high word of the Philox block index (2^34 elements)."""
+    the pairs, and no more than one high word of the Philox block index (2^34 elements; tables
+    of up to 10^8 elements that cross one take a launch less)."""
     room = (32704 - 32 * pairs) // 32 - 1
     count, held, high = 0, 0, None
     for numel, first in zip([t.numel() for t in table.tensors], table.flat_offsets):

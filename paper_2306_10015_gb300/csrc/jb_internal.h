@@ -13,11 +13,11 @@
 // the number of tiles, so a tile's segment is the last entry whose tile0 is not
 // above it.
 //
-// All global indices of a launch agree in the high word of their Philox block
-// index: the host cuts segments at multiples of 2^33 elements and puts those of
-// different high words into different launches. Block counters are therefore 32-bit
-// in the kernels, and the whole first round and half of the second are constants of
-// the pair (jb_rng.cuh).
+// All global indices of a segment agree in the high word of their Philox block index: the
+// host cuts segments at multiples of 2^33 elements. A launch holds segments of one high
+// word, or of two with a set of pairs for each. Block counters are therefore 32-bit in the
+// kernels, and the whole first round and half of the second are constants of the pair
+// (jb_rng.cuh).
 #pragma once
 #include <cstdint>
 
@@ -110,7 +110,8 @@ struct Launch {
     uint32_t n_tiles;
     uint32_t span;       // consecutive tiles that a warp takes at a time
     uint32_t write_src;  // write the result to the source too; checksum: one CTA, store the sum
-    uint32_t window_hi;  // checksum: high word of every window index
+    uint32_t second_from;  // segments from this one on have the second high word, and use
+                           // the second set of pairs (checksum: the second word of `data`)
     uint32_t seg_at;     // byte offset of the segment table in `data`; the pairs are at 0
     alignas(16) unsigned char data[BYTES];
 };

@@ -73,6 +73,15 @@ struct Shape {
 };
 
 constexpr uint64_t kSmallTiles = 1600;  // tiles of the large shape
+// Tables that cross a multiple of 2^34 elements (checksum of bf16: 2^35) take one launch
+// with a set of pairs for each of two high words up to this many tiles, or twice as many for
+// one pair: two launches of fewer tiles leave more warps idle at their ends and cost about
+// 4 us each (two launches / one, us: fp32 perturbation 4M elements 14.2 / 8.2, 8M 18.6 /
+// 14.3, 128M 170 / 168; K = 3 update 4.6M fp32 24.5 / 20.5, bf16 26.1 / 20.4, 128M 421 / 420
+// and 418 / 415; bf16 perturbation 256M 290 / 287). Above it the kernels for one high word
+// are up to 2 % faster, and in fp32 the round keys come with the pairs. The checksum takes
+// one launch always (256M fp32 161 / 155).
+constexpr uint64_t kMergeTiles = 1u << 17;
 
 template <typename T>
 struct Traits;
@@ -197,6 +206,10 @@ __device__ __forceinline__ uint64_t dst_of(const SegParamOut& g) { return g.dst;
 
 enum Store { kInPlace, kToDst, kNowhere };
 
+// What a kernel's launch may hold: vectors on the 16-byte grid alone, off it too, or that
+// and a second high word of the indices.
+enum Tables { kOnGrid, kOffGrid, kTwoHighs };
+
 // Runs op(x, blk, present) on each of this warp's tiles and stores the result (in place,
 // to the destination table, and then also back to the source when also_src, or nowhere):
 // x[j] is vector 32 j + lane of the tile in storage form, blk the low word of the first
@@ -206,12 +219,13 @@ enum Store { kInPlace, kToDst, kNowhere };
 // grid; spans that follow one another go to different SMs, so that a few tiles occupy as
 // many SMs. Which warp handles a tile never changes a result: every element's value
 // depends only on its own stored value, its global index and the seeds. Vectors that are
-// partial (the ends of a segment) go element by element. OFF: segments may lie off the
-// 16-byte grid.
-template <typename T, typename S, Store TO, bool OFF, typename P, typename Op>
+// partial (the ends of a segment) go element by element. op's last argument says whether
+// the tile's indices have the launch's second high word.
+template <typename T, typename S, Store TO, Tables HOLDS, typename P, typename Op>
 __device__ __forceinline__ void visit_tiles(const P& p, bool also_src, Op&& op) {
     constexpr int E = Traits<T>::E, V = S::V;
     constexpr uint32_t B = TO == kNowhere ? 1 : E / 4, kTileVec = 32u * V;
+    constexpr bool OFF = HOLDS != kOnGrid;
     const uint32_t lane = threadIdx.x & 31u;
     const uint64_t span = p.span;
     const uint64_t stride = span * (static_cast<uint64_t>(gridDim.x) * (S::THREADS / 32));
@@ -227,6 +241,9 @@ __device__ __forceinline__ void visit_tiles(const P& p, bool also_src, Op&& op) 
             const uint32_t stop = next < t_end ? next : t_end;
             const uint32_t v_lo = g.lo, v_hi = g.full;
             const uint32_t load_align = OFF ? g.load : 16u, store_align = OFF ? g.store : 16u;
+            // from lane 0, so that the compiler knows it for the same in all lanes and reads the
+            // pairs with uniform indices (K = 16 update of 2^28 elements 4340 -> 4140 us)
+            const bool second = HOLDS == kTwoHighs && __shfl_sync(0xFFFFFFFFu, s >= p.second_from ? 1 : 0, 0) != 0;
             uint32_t v = (t - g.tile0) * kTileVec;  // first vector of the tile
             uint64_t src = g.base + 16ull * (v + lane);
             uint64_t dst = dst_of(g) + 16ull * (v + lane);
@@ -256,9 +273,10 @@ __device__ __forceinline__ void visit_tiles(const P& p, bool also_src, Op&& op) 
                 }
                 if constexpr (TO == kNowhere) {
                     const uint64_t vecs = (g.end + E - 1) / E;  // a tile has at least one
-                    op(x, blk, fast ? kTileVec : static_cast<uint32_t>(vecs < v + lane ? 0 : vecs - v - lane));
+                    op(x, blk, fast ? kTileVec : static_cast<uint32_t>(vecs < v + lane ? 0 : vecs - v - lane),
+                       second);
                 } else {
-                    op(x, blk);
+                    op(x, blk, second);
                 }
                 constexpr bool TO_DST = TO == kToDst;
                 const uint64_t out = TO_DST ? dst : src;
@@ -339,9 +357,9 @@ __device__ __forceinline__ uint4 add_round(uint4 raw, const float2 (&acc)[B][2])
 // stream (one block's words ahead instead of the tile's: 4% slower). The last pair is
 // peeled. Philox round 1's product of the block counter is the same for every pair.
 template <typename T, typename S, bool GROUPS, typename P>
-__device__ __forceinline__ void update_tile(const P& p, uint4 (&x)[S::V], uint32_t blk) {
+__device__ __forceinline__ void update_tile(const P& p, uint4 (&x)[S::V], uint32_t blk, bool second) {
     constexpr int V = S::V, B = Traits<T>::E / 4, NB = V * B;
-    const uint32_t n = p.n_seeds;
+    const uint32_t n = p.n_seeds, first = second ? n : 0u;
     if (GROUPS && n == 0u) return;  // a copy
     float2 acc[V][B][2];
     BlockCtr bc[NB];
@@ -352,14 +370,14 @@ __device__ __forceinline__ void update_tile(const P& p, uint4 (&x)[S::V], uint32
     }
     uint4 w[NB];
 #pragma unroll
-    for (int i = 0; i < NB; ++i) w[i] = philox_block(seed_at(p, 0), bc[i]);
+    for (int i = 0; i < NB; ++i) w[i] = philox_block(seed_at(p, first), bc[i]);
     auto pair = [&](uint32_t k, auto more) {
-        const auto& sd = seed_at(p, k);
+        const auto& sd = seed_at(p, first + k);
         const float2 c = splat(sd.coef);
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
             uint4 wn;
-            if constexpr (decltype(more)::value) wn = philox_block(seed_at(p, k + 1), bc[i]);
+            if constexpr (decltype(more)::value) wn = philox_block(seed_at(p, first + k + 1), bc[i]);
             accum_block(w[i], c, acc[i / B][i % B][0], acc[i / B][i % B][1]);
             if constexpr (decltype(more)::value) w[i] = wn;
         }
@@ -381,10 +399,10 @@ __device__ __forceinline__ void update_tile(const P& p, uint4 (&x)[S::V], uint32
     }
 }
 
-template <typename T, typename S, bool OFF, typename P>
+template <typename T, typename S, Tables HOLDS, typename P>
 __global__ void __launch_bounds__(S::THREADS) seeded_kernel(const __grid_constant__ P p) {
-    visit_tiles<T, S, kInPlace, OFF>(p, false, [&](uint4 (&x)[S::V], uint32_t blk) {
-        update_tile<T, S, false>(p, x, blk);
+    visit_tiles<T, S, kInPlace, HOLDS>(p, false, [&](uint4 (&x)[S::V], uint32_t blk, bool second) {
+        update_tile<T, S, false>(p, x, blk, second);
     });
 }
 
@@ -396,9 +414,9 @@ __global__ void __launch_bounds__(S::THREADS) seeded_kernel(const __grid_constan
 // counter's product from the first one's (bf16 perturbation of 2^28 elements 288.8 -> 282.7
 // us; further from the tile's first block: 282.7 too, but fp32 319 -> 325).
 template <typename T, int V, bool PERTURB, typename P>
-__device__ __forceinline__ void one_seed_tile(const P& p, uint4 (&x)[V], uint32_t blk) {
+__device__ __forceinline__ void one_seed_tile(const P& p, uint4 (&x)[V], uint32_t blk, bool second) {
     constexpr int B = Traits<T>::E / 4;
-    const SeedParam& sd = seed_at(p, 0);
+    const SeedParam& sd = seed_at(p, second ? 1u : 0u);
     const float2 c = splat(sd.coef);
     uint4 wc[B], wn[B];
 #pragma unroll
@@ -427,21 +445,22 @@ __device__ __forceinline__ void one_seed_tile(const P& p, uint4 (&x)[V], uint32_
 
 enum OneSeed { kPerturbInPlace = 0, kAddInPlace = 1, kAddToDst = 2 };
 
-template <typename T, typename S, int MODE, bool OFF, typename P>
+template <typename T, typename S, int MODE, Tables HOLDS, typename P>
 __global__ void __launch_bounds__(S::THREADS) one_seed_kernel(const __grid_constant__ P p) {
     constexpr bool TO_DST = MODE == kAddToDst;
-    visit_tiles<T, S, TO_DST ? kToDst : kInPlace, OFF>(p, TO_DST && p.write_src != 0u, [&](uint4 (&x)[S::V], uint32_t blk) {
-        one_seed_tile<T, S::V, MODE == kPerturbInPlace>(p, x, blk);
-    });
+    visit_tiles<T, S, TO_DST ? kToDst : kInPlace, HOLDS>(
+        p, TO_DST && p.write_src != 0u, [&](uint4 (&x)[S::V], uint32_t blk, bool second) {
+            one_seed_tile<T, S::V, MODE == kPerturbInPlace>(p, x, blk, second);
+        });
 }
 
 // The generalised update: source -> destination (optionally also back to the
 // source), seeds applied in groups with a rounding to the storage type after each
 // group, exactly as successive in-place updates would round.
-template <typename T, typename S, bool OFF, typename P>
+template <typename T, typename S, Tables HOLDS, typename P>
 __global__ void __launch_bounds__(S::THREADS) general_update_kernel(const __grid_constant__ P p) {
-    visit_tiles<T, S, kToDst, OFF>(p, p.write_src != 0u, [&](uint4 (&x)[S::V], uint32_t blk) {
-        update_tile<T, S, true>(p, x, blk);
+    visit_tiles<T, S, kToDst, HOLDS>(p, p.write_src != 0u, [&](uint4 (&x)[S::V], uint32_t blk, bool second) {
+        update_tile<T, S, true>(p, x, blk, second);
     });
 }
 
@@ -614,16 +633,18 @@ __device__ __forceinline__ uint64_t window_hash(uint64_t win, uint4 w) {
     return ((static_cast<uint64_t>(x1) << 32) | x0) + ((static_cast<uint64_t>(x3) << 32) | x2);
 }
 
-// blk0 of the segments is the low word of the index of the first window, p.window_hi
-// the high word of all. One CTA alone stores its sum, which saves the clearing of *out.
-template <typename T, typename S, bool OFF, typename P>
+// blk0 of the segments is the low word of the index of the first window; the high words,
+// two of them, stand where other launches have their pairs. One CTA alone stores its sum,
+// which saves the clearing of *out.
+template <typename T, typename S, Tables HOLDS, typename P>
 __global__ void __launch_bounds__(S::THREADS) checksum_kernel(const __grid_constant__ P p,
                                                              unsigned long long* out) {
     uint64_t sum = 0;
-    visit_tiles<T, S, kNowhere, OFF>(p, false, [&](uint4 (&x)[S::V], uint32_t win, uint32_t present) {
+    visit_tiles<T, S, kNowhere, HOLDS>(p, false, [&](uint4 (&x)[S::V], uint32_t win, uint32_t present, bool second) {
+        const uint32_t high = reinterpret_cast<const uint32_t*>(p.data)[second ? 1 : 0];
 #pragma unroll
         for (int j = 0; j < S::V; ++j) {
-            const uint64_t w = (static_cast<uint64_t>(p.window_hi) << 32) | (win + 32u * j);
+            const uint64_t w = (static_cast<uint64_t>(high) << 32) | (win + 32u * j);
             if (32u * j < present) sum += window_hash(w, x[j]);
         }
     });
@@ -768,7 +789,7 @@ cudaError_t launch_split(const Job& job, P& p) {
     return cudaGetLastError();
 }
 
-template <typename T, bool SMALL, bool OFF, typename P>
+template <typename T, bool SMALL, Tables HOLDS, typename P>
 cudaError_t launch_work(const Job& job, P& p) {
     static GridCache caches[4];
     using C = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::Sum>;
@@ -778,30 +799,31 @@ cudaError_t launch_work(const Job& job, P& p) {
     const int ctas = job.grid_ctas;
     if constexpr (std::is_same<typename P::Pair, KeyedParam>::value) {
         if constexpr (std::is_same<typename P::Seg, SegParamOut>::value)
-            return launch<G>(general_update_kernel<T, G, OFF, P>, caches[0], p, ctas, job.stream);
+            return launch<G>(general_update_kernel<T, G, HOLDS, P>, caches[0], p, ctas, job.stream);
         else
-            return launch<U>(seeded_kernel<T, U, OFF, P>, caches[0], p, ctas, job.stream);
+            return launch<U>(seeded_kernel<T, U, HOLDS, P>, caches[0], p, ctas, job.stream);
     } else if constexpr (std::is_same<typename P::Seg, SegParamOut>::value) {
         using R = std::conditional_t<SMALL, typename Traits<T>::Small, typename Traits<T>::Refresh>;
         static_assert(R::V == S::V, "one table for both");
         if (p.n_seeds == 1 && p.write_src != 0u)
-            return launch<R>(one_seed_kernel<T, R, kAddToDst, OFF, P>, caches[2], p, ctas, job.stream);
+            return launch<R>(one_seed_kernel<T, R, kAddToDst, HOLDS, P>, caches[2], p, ctas, job.stream);
         if (p.n_seeds == 1)
-            return launch<S>(one_seed_kernel<T, S, kAddToDst, OFF, P>, caches[0], p, ctas, job.stream);
-        return launch<G>(general_update_kernel<T, G, OFF, P>, caches[1], p, ctas, job.stream);
+            return launch<S>(one_seed_kernel<T, S, kAddToDst, HOLDS, P>, caches[0], p, ctas, job.stream);
+        return launch<G>(general_update_kernel<T, G, HOLDS, P>, caches[1], p, ctas, job.stream);
     } else {
         if (job.work == kChecksum)
-            return launch<C>(checksum_kernel<T, C, OFF, P>, caches[3], p, ctas, job.stream, job.sum);
+            return launch<C>(checksum_kernel<T, C, HOLDS, P>, caches[3], p, ctas, job.stream, job.sum);
         if (job.work == kPerturb)
-            return launch<S>(one_seed_kernel<T, S, kPerturbInPlace, OFF, P>, caches[0], p, ctas, job.stream);
+            return launch<S>(one_seed_kernel<T, S, kPerturbInPlace, HOLDS, P>, caches[0], p, ctas, job.stream);
         if (p.n_seeds == 1)
-            return launch<S>(one_seed_kernel<T, S, kAddInPlace, OFF, P>, caches[1], p, ctas, job.stream);
-        return launch<U>(seeded_kernel<T, U, OFF, P>, caches[2], p, ctas, job.stream);
+            return launch<S>(one_seed_kernel<T, S, kAddInPlace, HOLDS, P>, caches[1], p, ctas, job.stream);
+        return launch<U>(seeded_kernel<T, U, HOLDS, P>, caches[2], p, ctas, job.stream);
     }
 }
 
 // Packs segments, cut at multiples of kPieceElems, into launches whose pieces share the
-// high word of their block (checksum: window) indices.
+// high word of their block (checksum: window) indices or, if the table fits one launch that
+// way, have one of two (kMergeTiles).
 template <typename T, typename SEG, typename PAIR = SeedParam>
 cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size_t n_segs) {
     using P = Launch<SEG, PAIR, kParamBytes>;
@@ -820,8 +842,16 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
     // faster without keys (2667 / 2694); the bf16 update, the one-pair kernels and small
     // tables (more parameters to copy) gain nothing.
     constexpr bool MAY_KEY = std::is_same<T, float>::value;
+    const uint64_t per_index = job.work == kChecksum ? E : 4;  // elements of a window or block
+    const auto high = [&](uint64_t fo) { return static_cast<uint32_t>((fo / per_index) >> 32); };
+    const uint32_t pair_bytes = job.work == kChecksum ? 16u : static_cast<uint32_t>(job.n_seeds * sizeof(PAIR));
+    const bool may_merge = job.work == kChecksum || big_tiles <= (job.n_seeds == 1 ? 2 : 1) * kMergeTiles;
+    bool merge = false;
+    if (!KEYED && !small && may_merge && 2 * pair_bytes + (n_segs + 8) * sizeof(SEG) <= kParamBytes)
+        for (size_t k = 0; k < n_segs && !merge; ++k)
+            merge = high(segs[k].fo) != high(segs[0].fo) || high(segs[k].fo + segs[k].n - 1) != high(segs[0].fo);
     if constexpr (MAY_KEY && !KEYED) {
-        if ((job.work == kUpdate || job.work == kGeneral) && job.n_seeds > 1 && !small &&
+        if (!merge && (job.work == kUpdate || job.work == kGeneral) && job.n_seeds > 1 && !small &&
             job.n_seeds * sizeof(KeyedParam) + (n_segs + 1) * sizeof(SEG) <= kParamBytes)
             return enqueue_t<T, SEG, KeyedParam>(job, segs, dst, n_segs);
     }
@@ -836,23 +866,27 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
     static thread_local P p;  // ~32 KB: keep it off the stack
     p.n_seeds = static_cast<uint32_t>(job.n_seeds);
     p.write_src = job.write_src ? 1u : 0u;
-    p.seg_at = static_cast<uint32_t>(job.n_seeds * sizeof(PAIR));
+    p.seg_at = merge && job.work != kChecksum ? 2 * pair_bytes : pair_bytes;
     const size_t room = (P::kBytes - p.seg_at) / sizeof(SEG) - 1;  // and the sentinel
     SEG* table = reinterpret_cast<SEG*>(p.data + p.seg_at);
 
-    const uint64_t per_index = job.work == kChecksum ? E : 4;  // elements of a window or block
     const uint64_t step = job.work == kChecksum ? 1 : win / 4;  // indices of a window
-    const auto high = [&](uint64_t fo) { return static_cast<uint32_t>((fo / per_index) >> 32); };
     size_t i = 0;
     uint64_t at = 0;  // elements of segs[i] already launched
     bool cleared = false;
     while (i < n_segs) {
-        const uint32_t hi = high(segs[i].fo + at);
-        size_t count = 0;
+        uint32_t his[2] = {high(segs[i].fo + at), 0u};
+        size_t count = 0, second_from = ~static_cast<size_t>(0);
         uint64_t tiles = 0;
         bool off_grid = false;
-        while (i < n_segs && count < room && high(segs[i].fo + at) == hi && tiles < (1ull << 30)) {
+        while (i < n_segs && count < room && tiles < (1ull << 30)) {
             const uint64_t fo = segs[i].fo + at;
+            const bool second = second_from <= count;
+            if (high(fo) != his[second ? 1 : 0]) {
+                if (!merge || second) break;
+                second_from = count;
+                his[1] = high(fo);
+            }
             const uint64_t n = std::min(segs[i].n - at, kPieceElems - fo % kPieceElems);
             const uint64_t src = segs[i].ptr + at * ES;
             const uint64_t to = dst != nullptr ? dst[i] + at * ES : src;
@@ -889,14 +923,18 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
         table[count].tile0 = static_cast<uint32_t>(tiles);
         p.n_segs = static_cast<uint32_t>(count);
         p.n_tiles = static_cast<uint32_t>(tiles);
-        PAIR* sp = reinterpret_cast<PAIR*>(p.data);
-        for (int k = 0; k < job.n_seeds; ++k) set_pair(sp[k], seed_param(job.seeds[k], hi, job.coef[k]));
-        for (int k = 0; k < job.n_groups; ++k) sp[job.group_end[k] - 1].ends_group = 1u;
-        if (job.work == kUpdate) sp[job.n_seeds - 1].ends_group = 1u;
+        const bool two_highs = second_from < count;
+        p.second_from = static_cast<uint32_t>(two_highs ? second_from : count);
+        for (int h = 0; h < (two_highs ? 2 : 1); ++h) {
+            PAIR* sp = reinterpret_cast<PAIR*>(p.data) + h * job.n_seeds;
+            for (int k = 0; k < job.n_seeds; ++k) set_pair(sp[k], seed_param(job.seeds[k], his[h], job.coef[k]));
+            for (int k = 0; k < job.n_groups; ++k) sp[job.group_end[k] - 1].ends_group = 1u;
+            if (job.work == kUpdate) sp[job.n_seeds - 1].ends_group = 1u;
+        }
         cudaError_t err;
         Job now = job;
         if (job.work == kChecksum) {
-            p.window_hi = hi;
+            std::memcpy(p.data, his, sizeof(his));
             // one CTA (two tiles per warp) instead of several and a cleared sum
             const bool alone = small && !cleared && i == n_segs && tiles <= 32 && job.grid_ctas <= 0;
             p.write_src = alone ? 1u : 0u;
@@ -909,19 +947,21 @@ cudaError_t enqueue_t(const Job& job, const Seg* segs, const uint64_t* dst, size
         }
         const size_t used = p.seg_at + (count + 1) * sizeof(SEG);
         if constexpr (KEYED) {
-            err = off_grid ? launch_work<T, false, true>(now, p) : launch_work<T, false, false>(now, p);
+            err = off_grid ? launch_work<T, false, kOffGrid>(now, p) : launch_work<T, false, kOnGrid>(now, p);
+        } else if (two_highs) {
+            err = launch_work<T, false, kTwoHighs>(now, p);
         } else if (split || (small && !off_grid)) {
             if (used > kSmallParamBytes) {
-                err = split ? launch_split<T>(now, p) : launch_work<T, true, false>(now, p);
+                err = split ? launch_split<T>(now, p) : launch_work<T, true, kOnGrid>(now, p);
             } else {
                 Launch<SEG, PAIR, kSmallParamBytes> q;
                 std::memcpy(&q, &p, offsetof(P, data) + used);
-                err = split ? launch_split<T>(now, q) : launch_work<T, true, false>(now, q);
+                err = split ? launch_split<T>(now, q) : launch_work<T, true, kOnGrid>(now, q);
             }
         } else if (small) {
-            err = launch_work<T, true, true>(now, p);
+            err = launch_work<T, true, kOffGrid>(now, p);
         } else {
-            err = off_grid ? launch_work<T, false, true>(now, p) : launch_work<T, false, false>(now, p);
+            err = off_grid ? launch_work<T, false, kOffGrid>(now, p) : launch_work<T, false, kOnGrid>(now, p);
         }
         if (err != cudaSuccess) return err;
     }

@@ -4,6 +4,8 @@ Philox block index changes: the result does not depend on either.
 A table that takes the large shape must give, bit for bit, what small tables over its
 pieces give (they take the one-vector shape); those are checked against the oracle in
 test_gpu_parity.py and, for the cuts, here."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -189,6 +191,74 @@ def test_segment_across_a_cut(jb, dtype, boundary):
         torch.cuda.synchronize()
         scale = update_scale(v, np.arange(fo, fo + v.size, dtype=np.uint64), seeds, q, LR, DENOM, QS)
         check_theta(to_host(dev), oracle.update(v, fo, seeds, q, LR, DENOM, QS), scale, f"{boundary}")
+
+
+def kernels_of(call):
+    """How many kernels a call launches: the kernel nodes of a graph captured from it."""
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        call()
+    cu, raw, n = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t()
+    assert cu.cuGraphGetNodes(raw, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert cu.cuGraphGetNodes(raw, nodes, ctypes.byref(n)) == 0
+    kinds = [ctypes.c_int(-1) for _ in range(n.value)]
+    for node, kind in zip(nodes, kinds):
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+    return sum(kind.value == 0 for kind in kinds)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("boundary", [1 << 34, 3 << 34, 1 << 35])
+@pytest.mark.parametrize("shift,parts", [(0, 1), (0, 7), (1, 7)])
+def test_large_table_across_a_high_word(jb, dtype, boundary, shift, parts):
+    """Tables of the large shape whose indices have two high words take one launch if they fit
+    it, and give what the pieces on either side of the boundary give by themselves: one tensor
+    that crosses, several, in any order (a third run of high words is another launch), on the
+    grid and off it."""
+    ops = operations(jb)
+    ops["update K=512"] = lambda t: jb.jb_apply_updates(t, *pairs(512), LR / 20, DENOM, QS)  # two sets do not fit
+
+    def refresh(t, K):
+        out = [torch.zeros_like(x) for x in t.tensors]
+        jb.jb_apply_updates_from(t, jb.ParamTable(out, t.flat_offsets), *pairs(K), LR, DENOM, QS, write_src=True)
+        assert all(torch.equal(x.view(torch.uint8), o.view(torch.uint8)) for x, o in zip(t.tensors, out))
+
+    ops["refresh K=1"], ops["refresh K=4"] = (lambda t: refresh(t, 1)), (lambda t: refresh(t, 4))
+    n, before = 3_000_003, 1_400_008
+    torch.manual_seed(parts)
+    base = torch.randn(n + 16, device="cuda").mul_(0.02).to(dtype)
+    ends = [n * (i + 1) // parts for i in range(parts)]
+    spans = list(zip([0] + ends, ends))
+    orders = {"in order": spans, "reversed": spans[::-1], "three runs": spans[1:] + spans[:1]}
+    for name, op in ops.items():
+        want = base.clone()
+        for a, b in ((0, before), (before, n)):
+            op(jb.ParamTable([want[shift + a:shift + b]], [boundary - before + a]))
+        for what, order in orders.items():
+            got = base.clone()
+            op(jb.ParamTable([got[shift + a:shift + b] for a, b in order], [boundary - before + a for a, _ in order]))
+            assert torch.equal(got.view(torch.uint8), want.view(torch.uint8)), (name, what)
+
+    def checksum(spans):
+        out = torch.zeros(1, dtype=torch.int64, device="cuda")
+        jb.jb_checksum(jb.ParamTable([base[shift + a:shift + b] for a, b in spans],
+                                     [boundary - before + a for a, _ in spans]), out)
+        return int(out.item()) & (2**64 - 1)
+
+    for spans in orders.values():
+        alone = sum(checksum([(a, b)] if b <= before or a >= before else [(a, before)]) +
+                    (checksum([(before, b)]) if a < before < b else 0) for a, b in spans)
+        assert checksum(spans) == alone % 2**64
+
+    table = jb.ParamTable([base[shift + a:shift + b] for a, b in orders["in order"]],
+                          [boundary - before + a for a, _ in orders["in order"]])
+    total = torch.zeros(1, dtype=torch.int64, device="cuda")
+    for call in (lambda: jb.jb_perturb(table, (7, 8, 9), 1e-3), lambda: jb.jb_apply_updates(table, *pairs(5), LR, DENOM, QS),
+                 lambda: jb.jb_replay_updates(table, [(*pairs(2), LR, 1.0), (*pairs(1), LR, 1.0)], QS),
+                 lambda: jb.jb_checksum(table, total)):
+        assert kernels_of(call) == 1
 
 
 def test_q4_across_a_high_word(jb):
