@@ -80,6 +80,30 @@ def test_large_shape_equals_small_pieces(jb, dtype, tiles, extra, shift):
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("count,largest,first", [(1700, 9, 3), (5000, 300, 0), (2500, 900, 5)])
+def test_thousands_of_tiny_tensors(jb, dtype, count, largest, first):
+    """Tables that take the large shape by their number of tensors, with tiles that are mostly
+    empty, in several launches, against one tensor over all of them."""
+    rng = np.random.default_rng(count)
+    ends = np.cumsum(rng.integers(1, largest + 1, count)).tolist()
+    spans = list(zip([0] + ends, ends))
+    n = ends[-1]
+    torch.manual_seed(count)
+    base = torch.randn(n, device="cuda").mul_(0.02).to(dtype)
+    for name, op in operations(jb).items():
+        whole, parts = base.clone(), base.clone()
+        op(jb.ParamTable([whole], [first]))
+        op(jb.ParamTable([parts[a:b] for a, b in spans], [first + a for a, _ in spans]))
+        assert torch.equal(whole.view(torch.uint8), parts.view(torch.uint8)), name
+    sums = [torch.zeros(1, dtype=torch.int64, device="cuda") for _ in range(2)]
+    starts = sorted({min((a + 7) // 8 * 8, n) for a, _ in spans} | {n})  # a window belongs to one tensor
+    cuts = list(zip(starts, starts[1:]))
+    jb.jb_checksum(jb.ParamTable([base], [8]), sums[0])
+    jb.jb_checksum(jb.ParamTable([base[a:b] for a, b in cuts], [8 + a for a, _ in cuts]), sums[1])
+    assert sums[0].item() == sums[1].item()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("n", [7, 33, 4099, 400_003, 1_700_021])
 def test_off_grid_equals_aligned(jb, dtype, n):
     """Tensors that start at every element of the 16-byte grid of their flat offsets (8, 4
