@@ -631,7 +631,7 @@ def run_e2e(a, jb, tensors, offs, seeds, codes, ghat, mids, own, stream, N, esiz
 
 
 # The sources the update kernel's device code and launch shape are built from.
-UPDATE_KERNEL_SOURCES = ("jb_internal.h", "jb_kernels.cu", "jb_rng.cuh")
+UPDATE_KERNEL_SOURCES = ("jb_internal.h", "jb_kernels.cu", "jb_offgrid.h", "jb_rng.cuh")
 
 
 def kernel_sources_digest() -> str:

@@ -47,7 +47,8 @@
  * layout). Recommended: flat_offset of tensor t = align_up(flat_offset of
  * t-1 + numel of t-1, 8) in named_parameters() order. The vectorised path
  * needs (ptr - flat_offset * sizeof(T)) to be a multiple of 16 bytes; other
- * segments are handled with smaller accesses, at lower speed.
+ * segments are handled with smaller accesses, at lower speed, and cost the
+ * others of the table up to 2 %.
  *
  * Arithmetic. z = s r in fp32, with r the radius and s the signed cosine or
  * sine of the element; |z| <= sqrt(48 ln 2) = 5.77. A scaled draw a z is formed

@@ -118,7 +118,8 @@ struct Launch {
 
 constexpr int kParamBytes = 32704;
 // Small launches: the parameters are copied for each launch (an empty kernel: 10.8 us
-// from call to end with 32 KB of them, 9.0 us with 4 KB).
+// from call to end with 32 KB of them, 9.0 us with 4 KB). Small tables off the 16-byte grid
+// have no kernels of their own for that and take the large ones.
 constexpr int kSmallParamBytes = 4064;
 static_assert(sizeof(Launch<SegParam, SeedParam, kParamBytes>) <= 32764, "launch exceeds the parameter space");
 

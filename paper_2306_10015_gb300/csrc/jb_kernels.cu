@@ -50,6 +50,8 @@ namespace {
 // memory, so the shapes differ by a few percent. Measured on 2^28 elements (us):
 //   update, K = 16   fp32 5 x 512: 4111 (4 x 512: 4147, 4 x 768: 4171, 6 x 512: 4156)
 //                    bf16 3 x 512: 4163 (2 x 512: 4332, 2 x 768: 4171, 2 x 640: 4156)
+//                    (at 128 registers a thread: bf16 3 x 512 spills 20 bytes of them, fp32
+//                    5 x 512 without round keys 12)
 //   replay, 10 pairs fp32 4 x 512: 2663 (4 x 768: 2871, 6 x 512: 2812)
 //                    bf16 2 x 512: 2667 (2 x 768: 2794, 3 x 512: 2817)
 //   one pair         fp32 4 x 1024: 318 (4 x 768: 338, 4 x 512: 329; HBM alone: 316)
@@ -63,9 +65,13 @@ namespace {
 // Small tables take one vector per thread in every kernel, and their launch fewer
 // parameter bytes: a scheduler needs about one warp's worth of blocks to be busy, so what
 // counts is that all 608 have some. The line lies where the large shape gives most of its
-// 16 warps per SM a tile (K = 32 update, us, one vector / large shape: fp32 512K elements
-// 27 / 29, 1M 43 / 39, 2M 84 / 76; bf16 256K 23 / 25, 512K 25 / 35, 1M 43 / 47, 1.5M 62 / 61,
-// 3M 111 / 104).
+// 16 warps per SM a tile (us, one vector / large shape: K = 32 update fp32 512K elements
+// 27 / 29, 1M 43 / 39, 2M 84 / 76; bf16 256K 14 / 25, 512K 25 / 35, 1M 43 / 47, 1.5M 62 / 61,
+// 3M 111 / 104; replay of 10 pairs fp32 512K 12 / 12, 1M 18 / 16, bf16 512K 11 / 13, 1M
+// 16 / 16; perturbation fp32 512K 4.8 / 6.2, 1M 4.8 / 6.3, 2M 8.2 / 6.2, bf16 1.5M 6.1 / 6.3,
+// 3M 8.2 / 7.5; checksum fp32 1M 6.2 / 7.2, 2M 7.9 / 7.7, bf16 2M 6.2 / 7.3, 4M 8.2 / 8.1).
+// It counts tiles, also those that short tensors leave mostly empty: 2000 tensors of 64 to
+// 800 elements take 83 to 152 us in the K = 32 update.
 template <int V_, int THREADS_, int UNROLL_, int CTAS_ = 0>
 struct Shape {
     static constexpr int V = V_, THREADS = THREADS_, UNROLL = UNROLL_;
@@ -142,7 +148,10 @@ __device__ __forceinline__ void store_vec(uint64_t a, uint4 w) { __stcs(reinterp
 // Memory for the vectors off the 16-byte grid of their flat offset (jb_offgrid.h). They
 // take kernels of their own (OFF; in the common ones the choice costs registers). One
 // perturbation of 2^28 elements, against element by element: bf16 295 us at 8 bytes, 306
-// at 4, 411 at 2 (541 to 615 before; 281 on the grid), fp32 350 and 368 (427; 317).
+// at 4, 410 at 2 (541 to 615 before; 281 on the grid), fp32 349 and 368 (427; 317). One such
+// tensor takes all of its launch there: 16 tensors of 2^28 elements on the grid and one of
+// 1000 off it, us, without and with that one: perturbation fp32 318 / 324, bf16 283 / 285,
+// K = 2 update 561 / 570 and 563 / 568, K = 16 4106 / 4125 and 4161 / 4160.
 struct Global {
     __device__ uint2 load64(uint64_t a) const { return __ldcs(reinterpret_cast<const uint2*>(a)); }
     __device__ uint32_t load32(uint64_t a) const { return __ldcs(reinterpret_cast<const uint32_t*>(a)); }
@@ -471,7 +480,8 @@ __global__ void __launch_bounds__(S::THREADS) general_update_kernel(const __grid
 // pair order, chunk c while the group forms chunk c + 1. The additions are those of
 // update_tile, so the results are the same bit for bit. One warp alone needs about 350
 // cycles per pair for a tile (the latency of the generator and the transform; 580 where a
-// thread has the two blocks of a bf16 vector); shared out, an SM needs about 40. K = 400
+// thread has the two blocks of a bf16 vector); shared out, an SM needs about 115, or 85 per
+// tile where it has three or four (40 is what the issue of their instructions takes). K = 400
 // update, us, without and with the split: fp32 1K to 19K elements 70 and 29, 65K 85 and 62,
 // 78K 85 and 96; bf16 1K 117 and 31, 65K 119 and 62, 131K 150 and 112, 160K 150 and 156,
 // 262K 150 and 222. So it ends at one tile per scheduler (608) in fp32 and at two in bf16.

@@ -143,11 +143,12 @@ __device__ __forceinline__ const SegParamQ4& q4_seg(const P& p, uint32_t s) {
 // A warp tile is 1024 consecutive elements of one tensor, 32 per lane; tiles and spans as
 // in the update's kernels. Bound, like those, by operand reads and the instruction mix
 // (151 instructions and 218 cycles per scheduler and four elements of a warp; FMA pipe 76%
-// busy, shared-memory reads 36%). Eight warps per scheduler at 64 registers, a few spilled: 2^28 elements in 358 us (768 threads 364, 640 threads 365, 512 threads 386);
-// 397 before, with lanes numbered across tensors, codes shifted into place and bank
-// conflicts on the buckets.
+// busy, shared-memory reads 36%). Eight warps per scheduler at 64 registers, 36 bytes of them
+// spilled: 2^28 elements in 358 us (768 threads 364, 640 threads 365, 512 threads 386). With
+// lanes numbered across tensors, codes shifted into place and bank conflicts on the buckets
+// it took 397.
 // ONE_HI: the pair's constants hold for every block of the launch; otherwise they are
-// formed for the high word of each block's own index.
+// formed for the high word of each block's own index (2^28 elements 358 -> 376 us).
 template <bool ONE_HI, typename P>
 __global__ void __launch_bounds__(kThreadsQ4) q4_perturb_kernel(const __grid_constant__ P p) {
     constexpr int E = kQ4Epl, NB = E / 4, NW = E / 8;
